@@ -291,7 +291,11 @@ typedef struct {
                             /* same with the next hop's records requested      */
                             /* early, 8 with the row's own records copied in   */
                             /* as well (FP32 and 16-bit storage; other shapes  */
-                            /* take tile[1] = 2);                              */
+                            /* take tile[1] = 2); 9 marches tiles of rows      */
+                            /* along z (FP32 and 16-bit storage): tile[0] =    */
+                            /* vectors per group (even), tile[2] = rows per    */
+                            /* tile | z segments << 8 | ring units << 16 (a    */
+                            /* shape that does not fit goes to the planner);   */
                             /* tile[2] (tile[1] = 6..8): each CTA requests     */
                             /* into L2 the W rows and records of the row       */
                             /* tile[2] planes ahead in launch order; 0 none,   */

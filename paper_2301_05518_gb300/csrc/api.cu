@@ -9,6 +9,7 @@
 #include <cstring>
 
 #include "api_internal.h"
+#include "col_plan.h"
 
 namespace tls {
 
@@ -153,6 +154,16 @@ cudaError_t launch_hop(const StepArgs &a)
     case P_F32: return launch_hop_f32(a);
     case P_F16: return launch_hop_f16(a);
     case P_BF16: return launch_hop_bf16(a);
+    default: return cudaErrorNotSupported;
+    }
+}
+
+cudaError_t launch_step_col(const StepArgs &a)
+{
+    switch (a.prec_in) {
+    case P_F32: return launch_step_col_f32(a);
+    case P_F16: return launch_step_col_f16(a);
+    case P_BF16: return launch_step_col_bf16(a);
     default: return cudaErrorNotSupported;
     }
 }
@@ -685,11 +696,12 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     const size_t io_elem = io_prec == TLS_F64 ? 8 : 4;
     const size_t io_slice_bytes = (size_t)Vslice * 6 * io_elem;
 
-    // Kernel choice: explicit kernel, or the autotune table, or the planner's default.
+    // Kernel choice: explicit kernel, or the autotune table, or the planner.
     int kern = kernel;
     int vb = 0;
     int threads = 0;
     int tile[3] = {0, 0, 0};
+    bool planned = true;
     {
         TuneKey key{{gg->L[0], gg->L[1], gg->L[2], gg->L[3]}, nsl, nvec, storage, gg->wfmt};
         auto it = ctx->tune.find(key);
@@ -701,15 +713,41 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
             vb = it->second.vb;
             threads = it->second.threads;
             for (int k = 0; k < 3; ++k) tile[k] = it->second.tile[k];
+            planned = false;
         }
     }
     if (force_vb > 0) vb = force_vb;
     if (force_threads > 0) threads = force_threads;
-    if (force_tile)
+    if (force_tile) {
         for (int k = 0; k < 3; ++k) tile[k] = force_tile[k];
+        planned = false;
+    }
     if (op == 1) {  // one-link hops: the interleaved kernel only
         kern = TLS_KERNEL_MRHS;
         for (int k = 0; k < 3; ++k) tile[k] = 0;
+        planned = false;
+    }
+    // The column kernel (tile[1] = 9) works on vector groups of tile[0], one interleaved field
+    // behind the other; a shape it does not take goes to the planner.
+    const bool col_ok = kern == TLS_KERNEL_MRHS && op == 0 && storage != TLS_F64;
+    const int col_n = std::min(nvec, 256);
+    ColPlan cp{};
+    bool col = false;
+    if (col_ok && tile[1] == 9) {
+        col = col_shape(g, nblk, col_n, VBY, wfmt_bytes(fmt), tile[0], tile[2] & 255, std::max(1, (tile[2] >> 8) & 255),
+                        cp);
+        planned = !col;
+    }
+    if (col_ok && planned) {
+        double us = 0;
+        const double row_us = row_estimate(g, nblk, col_n, VBY, wfmt_bytes(fmt));
+        if (col_plans(g, nblk, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1) && us < row_us) {
+            col = true;
+            col_tile_of(cp, tile);
+        } else {
+            vb = row_tile(g, nblk, col_n, VBY, tile);
+            threads = 0;
+        }
     }
     // FP32 and 16-bit records of the interleaved layout come in vector pairs:
     // a group of an odd number of vectors carries one padding record
@@ -749,12 +787,21 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     const bool staged = vecs_dev == nullptr;
 
     // Workspace.
-    size_t a_bytes = (size_t)vs * (il_layout ? rec_of(G) : G);
-    s = ensure(ctx, ctx->A, a_bytes, "tls_smear: vector buffer A");
-    if (s == TLS_OK) s = ensure(ctx, ctx->B, a_bytes, "tls_smear: vector buffer B");
+    auto packed_of = [&](int n) {  // records per site in the packed buffers
+        return col ? (n + cp.nvg - 1) / cp.nvg * cp.nvg : il_layout ? rec_of(n) : n;
+    };
+    s = ensure(ctx, ctx->A, (size_t)vs * packed_of(G), "tls_smear: vector buffer A");
+    if (s == TLS_OK) s = ensure(ctx, ctx->B, (size_t)vs * packed_of(G), "tls_smear: vector buffer B");
+    if (s != TLS_OK && col && packed_of(G) > rec_of(G)) {  // without the padding of the vector groups
+        col = false;
+        vb = row_tile(g, nblk, col_n, VBY, tile);
+        if (G0 % vb != 0) vb = default_il_vb(storage, G0);
+        s = ensure(ctx, ctx->A, (size_t)vs * packed_of(G), "tls_smear: vector buffer A");
+        if (s == TLS_OK) s = ensure(ctx, ctx->B, (size_t)vs * packed_of(G), "tls_smear: vector buffer B");
+    }
     // alpha per vector in FP64, then the same rounded to FP32 (read by the FP32-arithmetic
     // kernels); one more entry of each for a padding record
-    const int nalpha = nvec + 1;
+    const int nalpha = nvec + std::max(1, col ? cp.nvg : 0);
     const size_t alpha_bytes = sizeof(double) * nalpha + sizeof(float) * nalpha;
     if (s == TLS_OK) s = ensure(ctx, ctx->alpha, alpha_bytes, "tls_smear: alpha");
     if (s == TLS_OK && norms_out)
@@ -871,14 +918,19 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         const size_t io_vec_bytes = (size_t)vsites * 6 * io_elem_b;
         for (int g0 = 0; g0 < nvec && e == cudaSuccess; g0 += G) {
             const int gn = std::min(G, nvec - g0);
-            const int rn = il_layout ? rec_of(gn) : gn;  // records per site in the packed buffers
+            const int rn = packed_of(gn);
+            const int sub = col ? cp.nvg : gn;  // vectors per interleaved field
             const char *src_g = src_io + (size_t)g0 * io_vec_bytes;
             char *dst_g = dst_io + (size_t)g0 * io_vec_bytes;
             const bool il = il_layout;
             const int m0 = ev_rec(st);
-            e = il ? launch_pack_il(src_g, io_prec, vsites, (char *)ctx->A.p, storage, g, gg->L, t_rel0, ns, gn, rn, 0,
-                                    st)
-                   : launch_pack_vectors(src_g, io_prec, vsites, (char *)ctx->A.p, storage, vsg, g, gg->L, t_rel0, ns,
+            if (il) {
+                for (int v = 0; v < gn && e == cudaSuccess; v += sub)
+                    e = launch_pack_il(src_g + (size_t)v * io_vec_bytes, io_prec, vsites,
+                                       (char *)ctx->A.p + (size_t)v * vsg, storage, g, gg->L, t_rel0, ns,
+                                       std::min(sub, gn - v), col ? sub : rn, 0, st, col);
+            } else
+                e = launch_pack_vectors(src_g, io_prec, vsites, (char *)ctx->A.p, storage, vsg, g, gg->L, t_rel0, ns,
                                          gn, st);
             ++launches;
             const int m1 = ev_rec(st);
@@ -922,6 +974,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
                     sa.threads = threads;
                     sa.stream = st;
                     sa.err = ctx->d_err;
+                    sa.num_sms = ctx->num_sms;
                     sa.vstride_in = sa.vstride_out = vsg;
                     for (int k = 0; k < 3; ++k) sa.tile[k] = tile[k];
                     const int sub_groups = kern == TLS_KERNEL_SINGLE ? gn : 1;
@@ -935,6 +988,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
                             sa.alpha = alpha_g + gi;
                             sa.alphaf = alphaf_g + gi;
                             e = op == 1                         ? launch_hop(sa)
+                                : col                           ? launch_step_col(sa)
                                 : kern == TLS_KERNEL_MRHS_ROWS  ? launch_step_rows(sa, ctx->d_err)
                                 : kern == TLS_KERNEL_MRHS_ZM    ? launch_step_zm(sa)
                                 : il                            ? launch_step_il(sa)
@@ -948,8 +1002,12 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
             }
             const int m2 = ev_rec(st);
             if (e == cudaSuccess) {
-                e = il ? launch_unpack_il(result, storage, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn, rn, 0, st)
-                       : launch_unpack_vectors(result, storage, vsg, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn,
+                if (il) {
+                    for (int v = 0; v < gn && e == cudaSuccess; v += sub)
+                        e = launch_unpack_il(result + (size_t)v * vsg, storage, dst_g + (size_t)v * io_vec_bytes, io_prec,
+                                             vsites, g, gg->L, t_rel0, ns, std::min(sub, gn - v), col ? sub : rn, 0, st, col);
+                } else
+                    e = launch_unpack_vectors(result, storage, vsg, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn,
                                                nullptr, nullptr, st);
                 ++launches;
             }

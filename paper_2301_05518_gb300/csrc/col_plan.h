@@ -1,0 +1,194 @@
+// col_plan.h -- tile shapes and shared-memory geometry of the column kernel (k_col.cuh).
+#pragma once
+
+#include <stdint.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "tls_types.h"
+
+namespace tls {
+
+constexpr int kColMaxUnits = 6;
+constexpr int kColMaxThreads = 512;  // consumers and the producer warp: 16 warps of 128 registers
+
+TLS_HD inline int up16(int n) { return (n + 15) & ~15; }
+
+// W rows of a unit, wb bytes per matrix.  The 16-byte words come as boxes of all
+// planes of br rows (one tensor copy each): nb boxes for the ny rows of W_x, of
+// W_y and of W_z, and a one-row box for row y0 - 1 of W_y.  The remainder planes
+// come as four plain pieces (x; y halo row; y; z), each with 16 spare bytes for
+// its alignment.
+struct ColW {
+    int br, nb;                   // rows per box, boxes per direction
+    int boxB, haloB;              // their shared-memory bytes (128-byte aligned)
+    int oX, oYh, oY, oZ;          // box offsets in the unit
+    int oRx, oRyh, oRy, oRz;      // remainder pieces
+    int bytes;
+};
+
+inline ColW col_w_plan(int wb, int hx, int ny)
+{
+    auto up = [](int n) { return (n + 127) & ~127; };
+    const int nq = wb / 16, rem = wb % 16;
+    ColW w{};
+    w.br = 1;
+    for (int r = 2; r <= ny; ++r)
+        if (ny % r == 0 && r * hx * 2 <= 256) w.br = r;  // a box row holds at most 256 doubles
+    w.nb = ny / w.br;
+    w.boxB = up(nq * w.br * hx * 16);
+    w.haloB = up(nq * hx * 16);
+    w.oX = 0;
+    w.oYh = w.nb * w.boxB;
+    w.oY = w.oYh + w.haloB;
+    w.oZ = w.oY + w.nb * w.boxB;
+    w.oRx = w.oZ + w.nb * w.boxB;
+    const int p = rem ? up16(ny * hx * rem) + 16 : 0, h = rem ? up16(hx * rem) + 16 : 0;
+    w.oRyh = w.oRx + p;
+    w.oRy = w.oRyh + h;
+    w.oRz = w.oRy + p;
+    w.bytes = up(w.oRz + p);
+    return w;
+}
+
+// Shared-memory geometry of one tile shape (bytes).
+struct ColPlan {
+    int nvg, ny, nseg, threads;  // vectors per group, rows per tile, z' segments, consumer threads (whole warps)
+    int ngrp, nyt, ntile;
+    int units;                   // ring units
+    int recB, wB, smem;          // one unit's records, one unit's W rows, the CTA's total
+    ColW w;
+};
+
+// The tile shape: nvg vectors per group, ny rows, nseg segments.  False: no fit.
+inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int nvg, int ny, int nseg, ColPlan &out)
+{
+    ColPlan p{};
+    if (nvg < 2 || (nvg & 1) || ny < 1 || ny > g.hy || nseg < 1 || nseg > g.hz) return false;
+    p.nvg = nvg;
+    p.ngrp = (nvec + nvg - 1) / nvg;
+    p.nyt = (g.hy + ny - 1) / ny;
+    p.ny = (g.hy + p.nyt - 1) / p.nyt;
+    p.nseg = nseg;
+    const int64_t act = (int64_t)(nvg / 2) * p.ny * g.hx;
+    if (act > kColMaxThreads - 32) return false;
+    p.threads = (int)((act + 31) / 32 * 32);
+    const int64_t recB = (int64_t)(p.ny + 2) * g.hx * nvg * vby;
+    p.recB = (int)((recB + 127) / 128 * 128);
+    p.w = col_w_plan(wb, g.hx, p.ny);
+    p.wB = p.w.bytes;
+    if (g.hx > 128 || p.w.nb > 8) return false;
+    p.units = (int)((227 * 1024 - 128) / (p.recB + p.wB));
+    if (p.units < 3) return false;
+    if (p.units > kColMaxUnits) p.units = kColMaxUnits;
+    p.smem = 128 + p.units * (p.recB + p.wB);
+    const int64_t nt = (int64_t)p.ngrp * p.nyt * nseg * nblk;
+    if (nt > 0x7fffffff) return false;
+    p.ntile = (int)nt;
+    out = p;
+    return true;
+}
+
+// Estimated time of one step (us) of the column kernel with tile shape p, fitted to
+// 1100 measured (lattice, vectors, shape) points on a GB300 (within 10 % for most;
+// the shape it picks is within 5 % of the best one measured, except on lattices
+// whose step takes a few launches' time anyway).  A unit of the busiest SM takes the
+// largest of: the arithmetic, 356 + 650 w cycles for w consumer warps on one
+// scheduler; the copies, 36.5 bytes per cycle; and, with d units in flight, 1/d of
+// a copy's latency of 2350 cycles plus its transfer.  A tile of n planes takes n + 2
+// units; the whole cannot beat the memory.  A thread rebuilds W for one vector pair
+// only, so W formats that need arithmetic cost it more than the row kernel.
+inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby, int wb, int num_sms)
+{
+    const int warps = p.threads / 32;
+    int occ = 1;
+    while ((occ + 1) * (warps + 1) <= 16 && (occ + 1) * (p.smem + 1024) <= 228 * 1024) ++occ;
+    const int eff = std::min(occ, (p.ntile + num_sms - 1) / num_sms);
+    const double rounds = (p.ntile + num_sms * eff - 1) / (num_sms * eff);
+    const double fmt = wb == 72 ? 1.0 : wb == 48 || wb == 36 ? 1.15 : wb == 24 ? 1.4 : 4.0;
+    const double unit = p.recB + p.wB;
+    const double comp = (356 + 650.0 * ((warps * eff + 3) / 4)) * (vby == 16 ? 1.145 : 1.0) * fmt;
+    const double copy = eff * unit / 36.5, lat = (2350 + unit / 36.5) / (p.units - 2);
+    const double t = std::pow(std::pow(comp, 6) + std::pow(copy, 6) + std::pow(lat, 6), 1.0 / 6);
+    const double us = rounds * ((double)g.hz / p.nseg + 2) * t / 2060;
+    const double dram = (double)nblk * g.Vs * (3.0 * wb + 2.0 * vby * p.ngrp * p.nvg) / 6.4e6;
+    return std::max(us, dram) * (1 + (rounds > 1 ? 0.005 : 0.03) * (p.units - 3)) + 3.5;
+}
+
+// The same for the row kernel (k_ilt.cuh): 0.03 + 0.0105 n ns per site for n vectors
+// in fours (0.0125 n above 24), 0.02 + 0.015 n otherwise (48^3 x 32: 3 / 5 / 12 / 24 /
+// 72 vectors 224 / 394 / 578 / 1018 / 3510 us; 64^3 x 24: 8 / 24 vectors 595 / 1624
+// us), 1.75 times that where its TMA copies do not apply (50^3 x 16, 24 vectors: 884
+// us), with the arithmetic of the W formats shared by four vectors (24 vectors at
+// 48^3 x 32, row / column kernel: f32-18 1018 / 927, f32-12 1103 / 1065, f32-8 1699 /
+// above 2600, 16-bit vectors with f32-18 1203 / 1037, with f16-12 1393 / 1414 us).
+inline double row_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb)
+{
+    const int n = (nvec + 1) & ~1;
+    const double fmt = wb == 48 ? 1.08 : wb == 32 ? 1.65 : wb == 24 ? 1.15 : 1.0;
+    const double site = n % 4 ? 0.02 + 0.015 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
+    const bool tma = (g.hx * (wb % 16)) % 16 == 0;
+    return (double)nblk * g.Vs * site * 1e-3 * (tma ? 1.0 : 1.75) * (vby == 16 ? 1.2 : 1.0) * fmt + 4;
+}
+
+// The best tile shapes by that estimate, best first (at most `most`).  nvg divides
+// the vectors into equal groups with at most a third of padding.
+inline int col_plans(const SubGeom &g, int nblk, int nvec, int vby, int wb, int num_sms, ColPlan *best, double *us,
+                     int most)
+{
+    int n = 0;
+    const int n2 = (nvec + 1) & ~1;
+    for (int nvg = 2; nvg <= 24 && nvg <= n2; nvg += 2) {
+        if ((nvec + nvg - 1) / nvg * nvg * 3 > 4 * n2) continue;
+        for (int last = 0, nyt = 1; nyt <= g.hy; ++nyt) {
+            const int ny = (g.hy + nyt - 1) / nyt;
+            if (ny == last) continue;
+            last = ny;
+            for (int nseg = 1; nseg <= 4 && nseg * 4 <= g.hz; nseg *= 2)
+                for (int few = 0; few < 2; ++few) {
+                    ColPlan p;
+                    if (!col_shape(g, nblk, nvec, vby, wb, nvg, ny, nseg, p)) continue;
+                    if (few) {  // three units: more CTAs per SM
+                        p.units = 3;
+                        p.smem = 128 + 3 * (p.recB + p.wB);
+                    }
+                    const double e = col_estimate(p, g, nblk, vby, wb, num_sms);
+                    int at = n < most ? n++ : most - 1;
+                    if (at == most - 1 && n == most && best[at].nvg && us[at] <= e) continue;
+                    while (at > 0 && us[at - 1] > e) {
+                        best[at] = best[at - 1];
+                        us[at] = us[at - 1];
+                        --at;
+                    }
+                    best[at] = p;
+                    us[at] = e;
+                }
+        }
+    }
+    return n;
+}
+
+// tile[] of the tune entry for a shape: 9 selects the column kernel.
+inline void col_tile_of(const ColPlan &p, int tile[3])
+{
+    tile[0] = p.nvg;
+    tile[1] = 9;
+    tile[2] = p.ny | p.nseg << 8 | p.units << 16;
+}
+
+// Row kernel parameters without a tune entry: tile[], returns the vectors per thread.
+// More than 24 vectors go through CTAs of 24 where that divides them (72 vectors at
+// 48^3 x 24: 2.41 ms against 2.64 with 36 a CTA); rows are asked into L2 ahead (tile[2])
+// where a step's data do not stay there (64^3 x 24, 24 vectors: 1.61 against 1.64 ms;
+// 16^3 x 32, 2 vectors: 21 against 19 us).
+inline int row_tile(const SubGeom &g, int nblk, int nvec, int vby, int tile[3])
+{
+    const int n = (nvec + 1) & ~1;
+    tile[0] = n > 24 && n % 24 == 0 ? 24 : 0;
+    tile[1] = 6;
+    tile[2] = (double)nblk * g.Vs * (216.0 + 2.0 * vby * n) > 120e6 ? -1 : 0;
+    return n % 4 == 0 ? 4 : 2;
+}
+
+}  // namespace tls

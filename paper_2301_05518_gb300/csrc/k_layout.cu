@@ -243,10 +243,19 @@ __global__ void __launch_bounds__(256) k_reduce_norms(const double *__restrict__
     if (threadIdx.x == 0) norms[v] = red[0];
 }
 
+// Site i of an interleaved block, in units of rec_n * SB bytes: the colour
+// planes of the block, or (rc) of each x'-row, one row behind the other.
+template <int VP> __device__ __forceinline__ int64_t il_site(const SubGeom &g, int i, bool rc)
+{
+    if (!rc || !il_planes(VP)) return i;
+    const int row = i / g.hx;
+    return (int64_t)row * 2 * g.hx + i;
+}
+
 // Interleaved layout: CTA = (nvec, spb); threadIdx.x = vector, threadIdx.y = site.
 template <typename IO, int VP>
 __global__ void k_pack_il(const IO *__restrict__ src, int64_t svs, char *__restrict__ dst, SubGeom g, int Lx, int Ly,
-                          int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0)
+                          int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0, bool rc)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     if (s >= nsite) return;
@@ -264,13 +273,13 @@ __global__ void k_pack_il(const IO *__restrict__ src, int64_t svs, char *__restr
         val[k].re = (R)p[2 * k];
         val[k].im = (R)p[2 * k + 1];
     }
-    VRec<VP>::store(dst + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + (int64_t)i * rec_n * VRec<VP>::SB, g.Ps * rec_n,
-                    rec_v0 + v, val);
+    VRec<VP>::store(dst + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + il_site<VP>(g, i, rc) * rec_n * VRec<VP>::SB,
+                    (rc ? g.hx : g.Ps) * rec_n, rec_v0 + v, val);
 }
 
 template <typename IO, int VP>
 __global__ void k_unpack_il(const char *__restrict__ src, IO *__restrict__ dst, int64_t dvs, SubGeom g, int Lx,
-                            int Ly, int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0)
+                            int Ly, int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0, bool rc)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     if (s >= nsite) return;
@@ -282,8 +291,8 @@ __global__ void k_unpack_il(const char *__restrict__ src, IO *__restrict__ dst, 
     const int64_t site = (((int64_t)t * Lz + c.z) * Ly + c.y) * Lx + c.x;
     typedef typename VRec<VP>::R R;
     cpx<R> val[3];
-    VRec<VP>::load(src + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + (int64_t)i * rec_n * VRec<VP>::SB, g.Ps * rec_n,
-                   rec_v0 + v, val);
+    VRec<VP>::load(src + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + il_site<VP>(g, i, rc) * rec_n * VRec<VP>::SB,
+                   (rc ? g.hx : g.Ps) * rec_n, rec_v0 + v, val);
     IO *p = dst + ((int64_t)v * dvs + site) * 6;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -327,12 +336,13 @@ __global__ void __launch_bounds__(256) k_norm_partials(const IO *__restrict__ ba
 // thread and step.  to_smem selects the direction.
 template <int VP>
 __device__ __forceinline__ void row_copy(unsigned char *smr, const void *gbase, int b, int r, const SubGeom &g, int hx,
-                                         int rec_n, bool to_smem)
+                                         int rec_n, bool to_smem, bool rc)
 {
     constexpr int SB = VRec<VP>::SB;
-    const int segB = hx * rec_n * SB;  // one colour (or the whole row for 16-bit records)
-    const int nseg = il_planes(VP) ? 3 : 1;
+    const int nseg = il_planes(VP) && !rc ? 3 : 1;
+    const int segB = hx * rec_n * vfmt_bytes(VP) / nseg;  // one colour, or the whole row
     char *blk = (char *)gbase + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP);
+    if (rc) blk += (int64_t)r * rec_n * (vfmt_bytes(VP) - SB);
     for (int c = 0; c < nseg; ++c) {
         uint4 *gs = reinterpret_cast<uint4 *>(blk + ((int64_t)c * g.Ps + r) * rec_n * SB);
         uint4 *ss = reinterpret_cast<uint4 *>(smr + c * segB);
@@ -352,7 +362,7 @@ __device__ __forceinline__ void row_copy(unsigned char *smr, const void *gbase, 
 template <typename IO, int VP>
 __global__ void __launch_bounds__(256) k_unpack_rows(const char *__restrict__ src, IO *__restrict__ dst, int64_t dvs,
                                                      SubGeom g, int Lx, int Ly, int Lz, int t_first, int nvec,
-                                                     int rec_n, int rec_v0)
+                                                     int rec_n, int rec_v0, bool rc)
 {
     extern __shared__ __align__(16) unsigned char smr[];
     constexpr int VBY = vfmt_bytes(VP);
@@ -363,7 +373,7 @@ __global__ void __launch_bounds__(256) k_unpack_rows(const char *__restrict__ sr
     const int r = ((z >> 1) * g.hy + (y >> 1)) * hx;
     const int segB = hx * rec_n * VBY;
     // stage both x'-rows (all rec_n records) with 16-byte loads
-    for (int par = 0; par < 2; ++par) row_copy<VP>(smr + par * segB, src, ts * 8 + (sub0 | par), r, g, hx, rec_n, true);
+    for (int par = 0; par < 2; ++par) row_copy<VP>(smr + par * segB, src, ts * 8 + (sub0 | par), r, g, hx, rec_n, true, rc);
     __syncthreads();
     typedef typename VRec<VP>::R R;
     const int64_t site0 = (((int64_t)(t_first + ts) * Lz + z) * Ly + y) * Lx;
@@ -384,7 +394,7 @@ __global__ void __launch_bounds__(256) k_unpack_rows(const char *__restrict__ sr
 template <typename IO, int VP>
 __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, int64_t svs, char *__restrict__ dst,
                                                    SubGeom g, int Lx, int Ly, int Lz, int t_first, int nvec, int rec_n,
-                                                   int rec_v0)
+                                                   int rec_v0, bool rc)
 {
     extern __shared__ __align__(16) unsigned char smr[];
     constexpr int VBY = vfmt_bytes(VP);
@@ -397,7 +407,7 @@ __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, i
     const bool partial = nvec != rec_n;
     if (partial) {  // keep the records of the other slots: start from the current segments
         for (int par = 0; par < 2; ++par)
-            row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, true);
+            row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, true, rc);
         __syncthreads();
     }
     typedef typename VRec<VP>::R R;
@@ -416,7 +426,7 @@ __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, i
     }
     __syncthreads();
     for (int par = 0; par < 2; ++par)
-        row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, false);
+        row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, false, rc);
 }
 
 inline int spb_of(int nvec) { return std::max(1, 256 / nvec); }
@@ -563,15 +573,15 @@ cudaError_t launch_unpack_vectors(const char *src, int prec, int64_t src_vstride
 
 template <typename IO>
 static cudaError_t pack_il_io(const IO *src, int64_t svs, char *dst, int prec, const SubGeom &g, const int L[4],
-                              int t_first, int64_t nsite, int nvec, int rec_n, int rec_v0, cudaStream_t s)
+                              int t_first, int64_t nsite, int nvec, int rec_n, int rec_v0, bool rc, cudaStream_t s)
 {
     const int spb = spb_of(nvec);
     dim3 block(nvec, spb), grid(nblocks(nsite, spb));
     switch (prec) {
-    case P_F64: k_pack_il<IO, P_F64><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
-    case P_F32: k_pack_il<IO, P_F32><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
-    case P_F16: k_pack_il<IO, P_F16><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
-    case P_BF16: k_pack_il<IO, P_BF16><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
+    case P_F64: k_pack_il<IO, P_F64><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
+    case P_F32: k_pack_il<IO, P_F32><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
+    case P_F16: k_pack_il<IO, P_F16><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
+    case P_BF16: k_pack_il<IO, P_BF16><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
     default: return cudaErrorNotSupported;
     }
     return cudaGetLastError();
@@ -579,15 +589,15 @@ static cudaError_t pack_il_io(const IO *src, int64_t svs, char *dst, int prec, c
 
 template <typename IO>
 static cudaError_t unpack_il_io(const char *src, int prec, IO *dst, int64_t dvs, const SubGeom &g, const int L[4],
-                                int t_first, int64_t nsite, int nvec, int rec_n, int rec_v0, cudaStream_t s)
+                                int t_first, int64_t nsite, int nvec, int rec_n, int rec_v0, bool rc, cudaStream_t s)
 {
     const int spb = spb_of(nvec);
     dim3 block(nvec, spb), grid(nblocks(nsite, spb));
     switch (prec) {
-    case P_F64: k_unpack_il<IO, P_F64><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
-    case P_F32: k_unpack_il<IO, P_F32><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
-    case P_F16: k_unpack_il<IO, P_F16><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
-    case P_BF16: k_unpack_il<IO, P_BF16><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0); break;
+    case P_F64: k_unpack_il<IO, P_F64><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
+    case P_F32: k_unpack_il<IO, P_F32><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
+    case P_F16: k_unpack_il<IO, P_F16><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
+    case P_BF16: k_unpack_il<IO, P_BF16><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
     default: return cudaErrorNotSupported;
     }
     return cudaGetLastError();
@@ -603,7 +613,7 @@ bool rows_transpose_ok(const SubGeom &g, int rec_n, int prec, const int L[4])
 
 template <typename IO>
 static cudaError_t rows_io(bool pack, const void *src, int64_t svs, void *dst, int prec, const SubGeom &g,
-                           const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0, cudaStream_t s)
+                           const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0, bool rc, cudaStream_t s)
 {
     dim3 grid((unsigned)(L[1] * L[2]), nsl);
     const int smem = 2 * g.hx * rec_n * vfmt_bytes(prec);
@@ -611,10 +621,10 @@ static cudaError_t rows_io(bool pack, const void *src, int64_t svs, void *dst, i
     case P:                                                                                                         \
         if (pack)                                                                                                   \
             k_pack_rows<IO, P><<<grid, 256, smem, s>>>((const IO *)src, svs, (char *)dst, g, L[0], L[1], L[2],       \
-                                                      t_first, nvec, rec_n, rec_v0);                                \
+                                                      t_first, nvec, rec_n, rec_v0, rc);                                \
         else                                                                                                        \
             k_unpack_rows<IO, P><<<grid, 256, smem, s>>>((const char *)src, (IO *)dst, svs, g, L[0], L[1], L[2],     \
-                                                        t_first, nvec, rec_n, rec_v0);                              \
+                                                        t_first, nvec, rec_n, rec_v0, rc);                              \
         break;
     switch (prec) {
         TLS_ROWS_CASE(P_F64)
@@ -629,45 +639,45 @@ static cudaError_t rows_io(bool pack, const void *src, int64_t svs, void *dst, i
 
 cudaError_t launch_pack_il(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                            const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                           cudaStream_t s)
+                           cudaStream_t s, bool rc)
 {
     const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
     if (nsite == 0 || nvec == 0) return cudaSuccess;
     if (nvec > 256 || rec_v0 < 0 || rec_v0 + nvec > rec_n) return cudaErrorInvalidValue;
     if (rows_transpose_ok(g, rec_n, prec, L)) {
         if (io_prec == P_F64)
-            return rows_io<double>(true, src, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
+            return rows_io<double>(true, src, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
         if (io_prec == P_F32)
-            return rows_io<float>(true, src, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
+            return rows_io<float>(true, src, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
     }
     if (io_prec == P_F64)
         return pack_il_io<double>((const double *)src, src_vstride_sites, dst, prec, g, L, t_first, nsite, nvec, rec_n,
-                                  rec_v0, s);
+                                  rec_v0, rc, s);
     if (io_prec == P_F32)
         return pack_il_io<float>((const float *)src, src_vstride_sites, dst, prec, g, L, t_first, nsite, nvec, rec_n,
-                                 rec_v0, s);
+                                 rec_v0, rc, s);
     return cudaErrorNotSupported;
 }
 
 cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, int64_t dst_vstride_sites,
                              const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                             cudaStream_t s)
+                             cudaStream_t s, bool rc)
 {
     const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
     if (nsite == 0 || nvec == 0) return cudaSuccess;
     if (nvec > 256 || rec_v0 < 0 || rec_v0 + nvec > rec_n) return cudaErrorInvalidValue;
     if (rows_transpose_ok(g, rec_n, prec, L)) {
         if (io_prec == P_F64)
-            return rows_io<double>(false, src, dst_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
+            return rows_io<double>(false, src, dst_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
         if (io_prec == P_F32)
-            return rows_io<float>(false, src, dst_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
+            return rows_io<float>(false, src, dst_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
     }
     if (io_prec == P_F64)
         return unpack_il_io<double>(src, prec, (double *)dst, dst_vstride_sites, g, L, t_first, nsite, nvec, rec_n,
-                                    rec_v0, s);
+                                    rec_v0, rc, s);
     if (io_prec == P_F32)
         return unpack_il_io<float>(src, prec, (float *)dst, dst_vstride_sites, g, L, t_first, nsite, nvec, rec_n,
-                                   rec_v0, s);
+                                   rec_v0, rc, s);
     return cudaErrorNotSupported;
 }
 

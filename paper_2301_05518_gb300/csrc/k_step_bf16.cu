@@ -2,11 +2,13 @@
 #include "k_stencil.cuh"
 #include "k_rows.cuh"
 #include "k_hop.cuh"
+#include "k_col.cuh"
 
 namespace tls {
 
 cudaError_t launch_step_bf16(const StepArgs &a) { return step_dispatch<P_BF16>(a); }
 cudaError_t launch_step_il_bf16(const StepArgs &a) { return step_il_dispatch<P_BF16>(a); }
+cudaError_t launch_step_col_bf16(const StepArgs &a) { return col_dispatch<P_BF16>(a); }
 cudaError_t launch_step_zm_bf16(const StepArgs &a) { return step_zm_dispatch<P_BF16>(a); }
 cudaError_t launch_hop_bf16(const StepArgs &a) { return hop_dispatch<P_BF16>(a); }
 cudaError_t launch_step_rows_bf16(const StepArgs &a, int *err) { return rows_dispatch<P_BF16>(a, err); }

@@ -280,6 +280,12 @@ template <typename H, int NR> struct WFmtH {
     static constexpr int REM = (NR * 2) % 16;  // 4 or 8
     static __device__ __forceinline__ void load(const char *blk, int64_t Ps, int i, cpx<float> m[9])
     {
+        load_split(blk, Ps, blk + NQ * Ps * 16, i, m);
+    }
+    // the same with the remainder plane at `rem` instead of behind the 16-byte planes
+    static __device__ __forceinline__ void load_split(const char *blk, int64_t Ps, const char *rem, int i,
+                                                      cpx<float> m[9])
+    {
         const uint4 *q = reinterpret_cast<const uint4 *>(blk);
         uint32_t u[NR / 2];
 #pragma unroll
@@ -288,10 +294,10 @@ template <typename H, int NR> struct WFmtH {
             u[4 * k] = v.x; u[4 * k + 1] = v.y; u[4 * k + 2] = v.z; u[4 * k + 3] = v.w;
         }
         if constexpr (REM == 8) {
-            uint2 v = reinterpret_cast<const uint2 *>(blk + NQ * Ps * 16)[i];
+            uint2 v = reinterpret_cast<const uint2 *>(rem)[i];
             u[4 * NQ] = v.x; u[4 * NQ + 1] = v.y;
         } else {
-            u[4 * NQ] = reinterpret_cast<const uint32_t *>(blk + NQ * Ps * 16)[i];
+            u[4 * NQ] = reinterpret_cast<const uint32_t *>(rem)[i];
         }
 #pragma unroll
         for (int k = 0; k < NR / 2; ++k) {

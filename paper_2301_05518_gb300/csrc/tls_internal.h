@@ -30,6 +30,7 @@ struct StepArgs {
     int threads;           // threads per CTA (multiple of 32)
     int tile[3];           // interleaved kernel: sites per CTA along x', y', z' (0 = a strip along x')
     int *err;              // device error word (kernels with bounded waits); nullable for the others
+    int num_sms;           // of the device (persistent CTAs of the column kernel)
     cudaStream_t stream;
 };
 
@@ -76,6 +77,10 @@ inline bool onchip_plan(const SubGeom &g, int wfmt_bytes_, int scratch_bytes, in
 cudaError_t launch_step(const StepArgs &a);
 // Interleaved-layout multi-RHS step (nvec <= 256 vectors per record group).
 cudaError_t launch_step_il(const StepArgs &a);
+// The same step on the grouped layout, marching along z' (k_col.cuh).  tile[0] =
+// vectors per group, tile[2] = rows per tile | z' segments << 8 | ring units << 16 (0: as many
+// as fit).
+cudaError_t launch_step_col(const StepArgs &a);
 // The same step marching along z' with a register window (interleaved layout, active unused).
 cudaError_t launch_step_zm(const StepArgs &a);
 // One-link Gaussian smearing step psi + alpha H psi (interleaved layout; W = the link field).
@@ -98,6 +103,9 @@ cudaError_t launch_step_il_f64(const StepArgs &a);
 cudaError_t launch_step_il_f32(const StepArgs &a);
 cudaError_t launch_step_il_f16(const StepArgs &a);
 cudaError_t launch_step_il_bf16(const StepArgs &a);
+cudaError_t launch_step_col_f32(const StepArgs &a);
+cudaError_t launch_step_col_f16(const StepArgs &a);
+cudaError_t launch_step_col_bf16(const StepArgs &a);
 cudaError_t launch_step_zm_f64(const StepArgs &a);
 cudaError_t launch_hop_f64(const StepArgs &a);
 cudaError_t launch_hop_f32(const StepArgs &a);
@@ -135,13 +143,14 @@ cudaError_t launch_export_twolink(const char *W, int wfmt, double *out, const Su
 // Whether the interleaved pack/unpack use the row transposes (contiguous canonical rows).
 bool rows_transpose_ok(const SubGeom &g, int rec_n, int prec, const int L[4]);
 // Interleaved layout: rec_n <= 256 records per site, record (block, i, r).  Caller vector v
-// (0 <= v < nvec) goes to / comes from record rec_v0 + v.
+// (0 <= v < nvec) goes to / comes from record rec_v0 + v.  rc: the colour planes are
+// those of each x'-row instead of the block's, so that a row is contiguous (column kernel).
 cudaError_t launch_pack_il(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                            const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                           cudaStream_t s);
+                           cudaStream_t s, bool rc = false);
 cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, int64_t dst_vstride_sites,
                              const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                             cudaStream_t s);
+                             cudaStream_t s, bool rc = false);
 // FP64 |psi|^2 partial sums of nvec canonical vectors (vector v at base + v * vstride
 // sites), kNormPartsPerSlice per (vector, slice) over nsl slices of slice_sites sites:
 // partial (v, s, p) at partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].

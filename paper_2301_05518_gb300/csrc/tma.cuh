@@ -74,6 +74,25 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned b
         : "memory");
 }
 
+// The same to a shared-memory address.
+__device__ __forceinline__ void bulk_load_s(uint32_t dst, const void *src, unsigned bytes, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+        "r"(bytes), "r"(smem_addr(bar))
+        : "memory");
+}
+
+// Box of a 3-D tensor map -> shared memory (128-byte aligned), completion counted on `bar`.
+__device__ __forceinline__ void tensor_load_3d(uint32_t dst, const void *map, int x, int y, int z, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(dst),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
+        : "memory");
+}
+
 // Asks the memory system to bring a contiguous global segment (16-byte
 // aligned, a multiple of 16 bytes) into L2; no completion is tracked.
 __device__ __forceinline__ void l2_prefetch(const void *src, unsigned bytes)

@@ -10,6 +10,7 @@
 #include <cstring>
 
 #include "api_internal.h"
+#include "col_plan.h"
 
 namespace tls {
 
@@ -20,7 +21,7 @@ struct Cand {
     int tile[3];
 };
 
-std::vector<Cand> candidates(int nvec, int storage)
+std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, int num_sms)
 {
     // The kernels that won at some measured shape.  Measured and dropped (they
     // never won at any benchmarked shape): the register-capped and W-staged
@@ -33,6 +34,16 @@ std::vector<Cand> candidates(int nvec, int storage)
         c.push_back({TLS_KERNEL_SINGLE, 1, 256, {0, 0, 0}});
     }
     const int G = std::min(nvec, 256);
+    if (storage != TLS_F64) {  // the column kernel at the tile shapes its cost model ranks first
+        ColPlan best[4] = {};
+        double us[4];
+        const int n = col_plans(gg.g, nsl * 8, G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms, best, us, 4);
+        for (int k = 0; k < n; ++k) {
+            Cand cd{TLS_KERNEL_MRHS, 2, 0, {0, 0, 0}};
+            col_tile_of(best[k], cd.tile);
+            c.push_back(cd);
+        }
+    }
     const int G2 = storage != TLS_F64 ? (G + 1) & ~1 : G;  // FP32 and 16-bit records come in vector pairs
     for (int vb : {1, 2, 4}) {
         if (G2 % vb != 0 || (storage == TLS_F64 && vb > 2)) continue;
@@ -118,7 +129,7 @@ tls_status tls_autotune(tls_ctx *ctx, tls_gauge_id id, int nvec, int storage, in
     ctx->profiling = true;
     TuneVal win{0, 0, 0, {0, 0, 0}, 1e300};
     int n = 0;
-    for (const Cand &c : candidates(nvec, storage)) {
+    for (const Cand &c : candidates(nvec, storage, gg, nsl, ctx->num_sms)) {
         // one warm-up call, then the timed one
         s = smear_impl(ctx, id, tmp, io, 1, nvec, 1, 0.5, timeslice, storage, c.kernel, c.vb, c.threads, c.tile,
                        nullptr, nullptr);
