@@ -139,6 +139,158 @@ __global__ void k_build_twolink(const double2 *__restrict__ Up, char *__restrict
     }
 }
 
+// --------------------------------------------------------------------------
+// The product rounded to FP32 without the FP64 pipe.
+//
+// k_build_twolink is bound by the FP64 pipe, which runs at 1/75 of the FP32 FMA
+// rate here (64^3 x 96: 16.3 ms against 2.4 ms for its bytes).  This form gives
+// the same bits from FP32 arithmetic wherever that decides the rounding, and
+// takes the FP64 chain of k_build_twolink for the elements where it does not.
+//
+// Split: each double |v| <= 1.125 becomes v0 + v1 + v2 with v0 a multiple of
+// 2^-10, v1 of 2^-21 (|v1| <= 2^-11) and |v2| <= 1.5 * 2^-22, off by less than
+// 2^-45 (taken from the bits of the double: no FP64 instruction).
+// Products, six per real part, by the sum of the slice indices:
+//   S0 = sum a0 b0                       multiples of 2^-20 below 8: exact in FP32
+//   S1 = sum a0 b1 + a1 b0               multiples of 2^-31 below 2^-7: exact
+//   S2 = sum a0 b2 + a1 b1 + a2 b0 + a1 b2 + a2 b1   below 2^-17, 30 roundings of
+//                                        at most 2^-42 each
+// S0 + S1 is renormalised exactly to h + l (two-sum) and l += S2.  The error of
+// h + l (roundings of S2 and l, the split, a2 b2) and of the FP64 chain itself add
+// up to less than T = 2^-36, so when RN(h + (l - T)) == RN(h + (l + T)) every value
+// in between, the FP64 chain's among them, rounds to that float.  The rest (about
+// 0.3 % of the elements of random SU(3) links; all of a matrix with an entry above
+// 1.125, an infinity or a NaN) is recomputed.
+// A matrix costs about 660 packed FP32 and 550 integer instructions of a warp;
+// slices of A stay in registers, those of B are made column by column.
+// tls_build_twolink at 48^3 x 64 with the links released: 6.3 ms before, 3.5 ms now, of
+// which 1.1 ms is cudaFree of the links (about 0.7 ms are the bytes at the copy rate).
+// --------------------------------------------------------------------------
+struct Slices {
+    float2 s[3];  // (re, im) of the three slices
+};
+
+// The leading 24 bits of v (truncated) and the next 23: v = f + g up to 2^-46 |v|.
+__device__ __forceinline__ void split_bits(double v, float &f, float &g, unsigned &top)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const unsigned mag = hi & 0x7fffffffu, sign = hi & 0x80000000u;
+    top = max(top, mag);
+    const unsigned fb = ((mag - (896u << 20)) << 3) | (lo >> 29);
+    const unsigned base = ((fb & 0x7f800000u) - (23u << 23)) | sign;
+    const bool tiny = mag < ((1023u - 60u) << 20);  // below 2^-60: taken as zero
+    f = tiny ? 0.0f : __uint_as_float(fb | sign);
+    g = tiny ? 0.0f : __uint_as_float(base | ((lo >> 6) & 0x7fffffu)) - __uint_as_float(base);
+}
+
+__device__ __forceinline__ Slices split3(double2 v, unsigned &top)
+{
+    float2 f, g;
+    split_bits(v.x, f.x, g.x, top);
+    split_bits(v.y, f.y, g.y, top);
+    Slices o;
+    const float2 m0 = make_float2(12288.0f, 12288.0f), n0 = make_float2(-12288.0f, -12288.0f);  // 1.5 * 2^13: units of 2^-10
+    const float2 m1 = make_float2(6.0f, 6.0f), n1 = make_float2(-6.0f, -6.0f);                  // 1.5 * 2^2: units of 2^-21
+    const float2 neg = make_float2(-1.0f, -1.0f);
+    o.s[0] = __fadd2_rn(__fadd2_rn(f, m0), n0);
+    const float2 r = __ffma2_rn(o.s[0], neg, f);  // exact
+    o.s[1] = __fadd2_rn(__fadd2_rn(r, m1), n1);
+    o.s[2] = __fadd2_rn(__ffma2_rn(o.s[1], neg, r), g);
+    return o;
+}
+
+// ROWS = 3 (W f32-18) or 2 (f32-12: rows 1-2 are stored).
+template <int ROWS>
+__global__ void __launch_bounds__(128, 4) k_build_split(const double2 *__restrict__ Up, char *__restrict__ W, SubGeom g,
+                                                        int64_t total)
+{
+    constexpr int WB = ROWS == 3 ? wfmt_bytes(W_F32_18) : wfmt_bytes(W_F32_12);
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= total) return;
+    const int i = (int)(idx % g.Vs);
+    const int64_t rr = idx / g.Vs;
+    const int d = (int)(rr % 3);
+    const int b = (int)(rr / 3);
+    const int sub = b & 7;
+    int fw[3], bw[3];
+    sub_neighbours(g, i, fw, bw);
+    const int ip = ((sub >> d) & 1) ? fw[d] : i;
+    const int bp = (b & ~7) | (sub ^ (1 << d));
+    const double2 *A = Up + ((int64_t)b * 3 + d) * 9 * g.Ps + i;
+    const double2 *B = Up + ((int64_t)bp * 3 + d) * 9 * g.Ps + ip;
+    unsigned top = 0;
+    Slices a[ROWS * 3];
+#pragma unroll
+    for (int k = 0; k < ROWS * 3; ++k) a[k] = split3(A[k * g.Ps], top);
+    float w[ROWS * 6];
+    unsigned bad = 0;
+    const float T = 1.0f / 68719476736.0f;  // 2^-36
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        float2 s[ROWS][3];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) s[r][q] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const Slices y = split3(B[(k * 3 + c) * g.Ps], top);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float2 p = y.s[j], t = make_float2(-p.y, p.x);  // i p
+#pragma unroll
+                for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if (q + j > 3) continue;
+                        const float2 x = a[r * 3 + k].s[q];
+                        float2 &acc = s[r][q + j > 2 ? 2 : q + j];
+                        acc = __ffma2_rn(make_float2(x.x, x.x), p, acc);
+                        acc = __ffma2_rn(make_float2(x.y, x.y), t, acc);
+                    }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const float2 neg = make_float2(-1.f, -1.f);
+            const float2 h = __fadd2_rn(s[r][0], s[r][1]);
+            const float2 v = __ffma2_rn(s[r][0], neg, h);  // two-sum: l = (S0 - (h - v)) + (S1 - v)
+            const float2 u = __ffma2_rn(v, neg, h);
+            float2 l = __fadd2_rn(__ffma2_rn(u, neg, s[r][0]), __ffma2_rn(v, neg, s[r][1]));
+            l = __fadd2_rn(l, s[r][2]);
+            const float2 up = __fadd2_rn(h, __fadd2_rn(l, make_float2(T, T)));
+            const float2 dn = __fadd2_rn(h, __fadd2_rn(l, make_float2(-T, -T)));
+            const int e = 2 * (r * 3 + c);
+            w[e] = up.x;
+            w[e + 1] = up.y;
+            bad |= (up.x == dn.x ? 0u : 1u << e) | (up.y == dn.y ? 0u : 2u << e);
+        }
+    }
+    if (top > 0x3FF20000u) bad = (1u << (6 * ROWS)) - 1u;  // an entry above 1.125
+    char *blk = W + ((int64_t)b * 3 + d) * g.Ps * WB;
+    float4 *q4 = reinterpret_cast<float4 *>(blk);
+#pragma unroll
+    for (int k = 0; k < ROWS * 6 / 4; ++k)
+        q4[k * g.Ps + i] = make_float4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+    if constexpr (ROWS == 3) reinterpret_cast<float2 *>(blk + 4 * g.Ps * 16)[i] = make_float2(w[16], w[17]);
+    while (bad) {  // undecided elements: the FP64 chain of k_build_twolink
+        const int e = __ffs(bad) - 1;
+        bad &= bad - 1;
+        const int r = e / 6, c = (e - 6 * r) >> 1;
+        double acc = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const double2 x = A[(r * 3 + k) * g.Ps], y = B[(k * 3 + c) * g.Ps];
+            acc = (e & 1) ? fma(x.x, y.y, acc) : fma(x.x, y.x, acc);
+            acc = (e & 1) ? fma(x.y, y.x, acc) : fma(-x.y, y.y, acc);
+        }
+        const float f = __double2float_rn(acc);
+        if (e < 16)
+            reinterpret_cast<float *>(q4 + (e >> 2) * g.Ps + i)[e & 3] = f;
+        else
+            reinterpret_cast<float *>(blk + 4 * g.Ps * 16)[2 * i + (e & 1)] = f;
+    }
+}
+
 template <int WF>
 __global__ void k_export_twolink(const char *__restrict__ W, double *__restrict__ out, SubGeom g, int Lx, int Ly,
                                  int Lz, int64_t total)
@@ -492,8 +644,8 @@ cudaError_t launch_build_twolink(const double *Up, char *W, int wfmt, const SubG
     const unsigned nb = nblocks(total, 128);
     switch (wfmt) {
     case W_F64_18: k_build_twolink<W_F64_18><<<nb, 128, 0, s>>>(u, W, g, total, err); break;
-    case W_F32_18: k_build_twolink<W_F32_18><<<nb, 128, 0, s>>>(u, W, g, total, err); break;
-    case W_F32_12: k_build_twolink<W_F32_12><<<nb, 128, 0, s>>>(u, W, g, total, err); break;
+    case W_F32_18: k_build_split<3><<<nb, 128, 0, s>>>(u, W, g, total); break;
+    case W_F32_12: k_build_split<2><<<nb, 128, 0, s>>>(u, W, g, total); break;
     case W_F32_8: k_build_twolink<W_F32_8><<<nb, 128, 0, s>>>(u, W, g, total, err); break;
     case W_F16_18: k_build_twolink<W_F16_18><<<nb, 128, 0, s>>>(u, W, g, total, err); break;
     case W_F16_12: k_build_twolink<W_F16_12><<<nb, 128, 0, s>>>(u, W, g, total, err); break;
