@@ -371,7 +371,8 @@ tls_status tls_load_gauge(tls_ctx *ctx, const double *U, int nd, const int dims[
     gg.Up_bytes = (size_t)dims[3] * 8 * 3 * 9 * gg.g.Ps * 16;
     tls_status s = dev_alloc(ctx, (void **)&gg.Up, gg.Up_bytes, "tls_load_gauge: packed links");
     if (s != TLS_OK) return s;
-    cudaError_t e = cudaMemsetAsync(gg.Up, 0, gg.Up_bytes, st);
+    // the padding sites between Vs and Ps are never read: no field is cleared
+    cudaError_t e = cudaSuccess;
     const int64_t Vslice = (int64_t)dims[0] * dims[1] * dims[2];
     const void *U_dev = on_device ? (const void *)U : nullptr;
     if (e == cudaSuccess && U_dev) {
@@ -449,7 +450,6 @@ tls_status tls_build_twolink(tls_ctx *ctx, tls_gauge_id id, int wprec, int recon
         tls_status s = dev_alloc(ctx, (void **)&gg->W, wbytes, "tls_build_twolink: W");
         if (s != TLS_OK) return s;
         gg->W_bytes = wbytes;
-        cudaMemsetAsync(gg->W, 0, wbytes, st);
     }
     cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
     if (ctx->profiling) cudaEventRecord(ctx->ev[0], st);
@@ -502,8 +502,7 @@ tls_status tls_ape_smear(tls_ctx *ctx, tls_gauge_id id, double alpha, int n_step
     double *tmp = nullptr;
     tls_status s = dev_alloc(ctx, (void **)&tmp, gg->Up_bytes, "tls_ape_smear: link copy");
     if (s != TLS_OK) return s;
-    cudaError_t e = cudaMemsetAsync(tmp, 0, gg->Up_bytes, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
+    cudaError_t e = cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
     if (ctx->profiling) cudaEventRecord(ctx->ev[0], st);
     double *cur = gg->Up, *nxt = tmp;
     const int nblk = gg->L[3] * 8;
@@ -555,7 +554,6 @@ tls_status tls_build_links(tls_ctx *ctx, tls_gauge_id id, int prec, int keep_U, 
         tls_status s = dev_alloc(ctx, (void **)&gg->L1, bytes, "tls_build_links: link field");
         if (s != TLS_OK) return s;
         gg->L1_bytes = bytes;
-        cudaMemsetAsync(gg->L1, 0, bytes, st);
     }
     cudaError_t e = launch_build_links(gg->Up, gg->L1, fmt, gg->g, gg->L[3] * 8, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
