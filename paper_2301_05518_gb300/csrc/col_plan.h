@@ -133,14 +133,14 @@ inline double row_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb
 }
 
 // The best tile shapes by that estimate, best first (at most `most`).  nvg divides
-// the vectors into equal groups with at most a third of padding.
+// the vectors into equal groups with at most a third of padding (exact: none).
 inline int col_plans(const SubGeom &g, int nblk, int nvec, int vby, int wb, int num_sms, ColPlan *best, double *us,
-                     int most)
+                     int most, bool exact = false)
 {
     int n = 0;
     const int n2 = (nvec + 1) & ~1;
     for (int nvg = 2; nvg <= 24 && nvg <= n2; nvg += 2) {
-        if ((nvec + nvg - 1) / nvg * nvg * 3 > 4 * n2) continue;
+        if ((nvec + nvg - 1) / nvg * nvg * 3 > 4 * n2 || (exact && nvec % nvg)) continue;
         for (int last = 0, nyt = 1; nyt <= g.hy; ++nyt) {
             const int ny = (g.hy + nyt - 1) / nyt;
             if (ny == last) continue;
@@ -181,14 +181,17 @@ inline void col_tile_of(const ColPlan &p, int tile[3])
 // More than 24 vectors go through CTAs of 24 where that divides them (72 vectors at
 // 48^3 x 24: 2.41 ms against 2.64 with 36 a CTA); rows are asked into L2 ahead (tile[2])
 // where a step's data do not stay there (64^3 x 24, 24 vectors: 1.61 against 1.64 ms;
-// 16^3 x 32, 2 vectors: 21 against 19 us).
+// 16^3 x 32, 2 vectors: 21 against 19 us).  Four vectors per thread where the rows then still
+// fill a warp (32^3 x 64 / 48^3 x 32, 3 vectors: 16 / 24 threads, 180 / 224 us with four and
+// 142 / 290 with two); 16-bit records want twice the threads (12 vectors, 48 threads: 434
+// against 369 us; 24 vectors, 144 threads: 1203 against 1507).
 inline int row_tile(const SubGeom &g, int nblk, int nvec, int vby, int tile[3])
 {
     const int n = (nvec + 1) & ~1;
     tile[0] = n > 24 && n % 24 == 0 ? 24 : 0;
     tile[1] = 6;
     tile[2] = (double)nblk * g.Vs * (216.0 + 2.0 * vby * n) > 120e6 ? -1 : 0;
-    return n % 4 == 0 ? 4 : 2;
+    return n % 4 == 0 && n / 4 * g.hx >= (vby == 16 ? 64 : 20) ? 4 : 2;
 }
 
 }  // namespace tls

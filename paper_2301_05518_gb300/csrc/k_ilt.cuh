@@ -584,6 +584,13 @@ __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict_
     const int blk = blockIdx.z / g.hz;
     const int zq = blockIdx.z - blk * g.hz;
     const bool leader = threadIdx.x == 0 && threadIdx.y == 0;
+    if constexpr (ACT) {  // serving: nothing to do for a vector group without an active slot
+        const int t = blockIdx.x * blockDim.x + threadIdx.x;
+        bool any = false;
+#pragma unroll
+        for (int v = 0; v < VB; ++v) any = any || active[il_vec<VP, VB>(t, nvec / VB, v)] != 0;
+        if (!__syncthreads_or(any)) return;
+    }
     // Only the leader touches the mbarrier (initialises it, issues the copies
     // and waits), so no CTA barrier is needed before the copies start.
     if (leader) {

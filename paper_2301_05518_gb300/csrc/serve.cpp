@@ -24,6 +24,7 @@
 #include <deque>
 
 #include "api_internal.h"
+#include "col_plan.h"
 
 namespace tls {
 
@@ -74,6 +75,8 @@ struct Batch {
     cudaStream_t stream = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool launched = false;
+    bool col = false;        // column kernel: slots in groups of cp.nvg, one interleaved field behind the other
+    ColPlan cp{};
     int *d_err = nullptr;    // device error word of this batch's kernels (bounded waits)
     int *h_err = nullptr;    // pinned copy, read after each round
 
@@ -146,6 +149,15 @@ tls_status make_batch(tls_ctx *ctx, Server *sv, const BatchKey &key, const Gauge
     b->S = batch_slots(key.storage, sv->opts.max_slots);
     b->K = sv->opts.steps_per_launch;
     b->vb = default_il_vb(key.storage, b->S);
+    if (key.storage != TLS_F64) {
+        // The column kernel skips slot groups without an active slot (so does the row kernel, by
+        // its larger CTA groups); it is taken unless the row kernel is clearly faster with every
+        // slot active.  Its groups divide the slots, so the buffers are the same size.
+        const int nb = (key.timeslice < 0 ? gg.L[3] : 1) * 8, vby = vfmt_bytes(key.storage), wb = wfmt_bytes(gg.wfmt);
+        double us = 0;
+        b->col = col_plans(gg.g, nb, b->S, vby, wb, ctx->num_sms, &b->cp, &us, 1, true) > 0 &&
+                 us < 1.1 * row_estimate(gg.g, nb, b->S, vby, wb);
+    }
     b->nsl = key.timeslice < 0 ? gg.L[3] : 1;
     b->t_first = key.timeslice < 0 ? 0 : key.timeslice;
     b->nblk = b->nsl * 8;
@@ -177,6 +189,28 @@ tls_status make_batch(tls_ctx *ctx, Server *sv, const BatchKey &key, const Gauge
     *out = b.get();
     sv->batches[key] = std::move(b);
     return TLS_OK;
+}
+
+// Packs the caller's n vectors into slots s0.. of the batch's current buffer, or unpacks
+// slots s0.. of buffer `buf` to the caller's layout; `v` is the canonical data, svs its
+// vector stride in sites.
+cudaError_t move_slots(const Batch &b, const Gauge &gg, bool pack, char *v, int io_prec, int64_t svs, int t_rel, int n,
+                       int s0, char *buf)
+{
+    const int per = b.col ? b.cp.nvg : b.S;  // slots of one interleaved field
+    const size_t vec_b = (size_t)svs * 6 * io_elem(io_prec);
+    for (int s = s0; s < s0 + n;) {
+        const int off = s % per, m = std::min(s0 + n - s, per - off);
+        char *field = buf + (size_t)(s - off) * b.vs;
+        char *x = v + (size_t)(s - s0) * vec_b;
+        const cudaError_t e =
+            pack ? launch_pack_il(x, io_prec, svs, field, b.key.storage, gg.g, gg.L, t_rel, b.nsl, m, per, off, b.stream, b.col)
+                 : launch_unpack_il(field, b.key.storage, x, io_prec, svs, gg.g, gg.L, t_rel, b.nsl, m, per, off, b.stream,
+                                    b.col);
+        if (e != cudaSuccess) return e;
+        s += m;
+    }
+    return cudaSuccess;
 }
 
 int find_slots(const Batch &b, int n)
@@ -281,8 +315,8 @@ int try_admit(tls_ctx *ctx, Server *sv, Job *j)
         svs = Vslice * b->nsl;
         t_rel = 0;
     }
-    cudaError_t e = launch_pack_il(src, j->d.io_prec, svs, b->buf[b->cur], j->d.storage, gg.g, gg.L, t_rel, b->nsl,
-                                   j->d.nvec, b->S, s0, b->stream);
+    cudaError_t e = move_slots(*b, gg, true, const_cast<char *>(src), j->d.io_prec, svs, t_rel, j->d.nvec, s0,
+                               b->buf[b->cur]);
     if (e != cudaSuccess) {
         finish(sv, j, cuda_fail(e, "serve: pack"));
         return 0;
@@ -326,10 +360,14 @@ cudaError_t launch_round(tls_ctx *ctx, Server *sv, Batch *b)
     sa.prec_in = sa.prec_out = b->key.storage;
     sa.vb = b->vb;
     sa.threads = 128;
-    // FP32 and 16-bit batches: whole-row CTAs with the W rows staged by TMA and
-    // vector-pair arithmetic (the packed kernel where the row shape does not
-    // allow it); FP64 batches use the plain interleaved kernel
-    if (b->key.storage != TLS_F64) sa.tile[1] = 6;
+    // FP32 and 16-bit batches: the column kernel, or whole-row CTAs with the W rows
+    // staged by TMA (the packed kernel where the row shape does not allow it); FP64
+    // batches use the plain interleaved kernel
+    if (b->col)
+        col_tile_of(b->cp, sa.tile);
+    else if (b->key.storage != TLS_F64)
+        sa.tile[1] = 6;
+    sa.num_sms = ctx->num_sms;
     sa.err = b->d_err;
     const float *d_alphaf = reinterpret_cast<const float *>(b->d_alpha + (size_t)b->K * b->S);
     sa.stream = b->stream;
@@ -340,7 +378,7 @@ cudaError_t launch_round(tls_ctx *ctx, Server *sv, Batch *b)
             sa.alpha = b->d_alpha + (size_t)j * b->S;
             sa.alphaf = d_alphaf + (size_t)j * b->S;
             sa.active = b->d_active + (size_t)j * b->S;
-            cudaError_t r = launch_step_il(sa);
+            cudaError_t r = b->col ? launch_step_col(sa) : launch_step_il(sa);
             if (r != cudaSuccess) return r;
         }
         return cudaSuccess;
@@ -396,11 +434,10 @@ void retire(tls_ctx *ctx, Server *sv, Batch *b)
         const size_t slice_b = (size_t)Vslice * 6 * io_elem(j->d.io_prec);
         cudaError_t e;
         if (j->d.vecs_on_device) {
-            e = launch_unpack_il(b->buf[j->parity], b->key.storage, j->d.vecs, j->d.io_prec, V, gg.g, gg.L, b->t_first,
-                                 b->nsl, j->d.nvec, b->S, s, b->stream);
+            e = move_slots(*b, gg, false, (char *)j->d.vecs, j->d.io_prec, V, b->t_first, j->d.nvec, s, b->buf[j->parity]);
         } else {
-            e = launch_unpack_il(b->buf[j->parity], b->key.storage, j->staging, j->d.io_prec, Vslice * b->nsl, gg.g,
-                                 gg.L, 0, b->nsl, j->d.nvec, b->S, s, b->stream);
+            e = move_slots(*b, gg, false, (char *)j->staging, j->d.io_prec, Vslice * b->nsl, 0, j->d.nvec, s,
+                           b->buf[j->parity]);
             const size_t width = slice_b * b->nsl, pitch = (size_t)V * 6 * io_elem(j->d.io_prec);
             if (e == cudaSuccess)
                 e = cudaMemcpy2DAsync((char *)j->d.vecs + (size_t)b->t_first * slice_b, pitch, j->staging, width,
