@@ -973,6 +973,8 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
                     sa.stream = st;
                     sa.err = ctx->d_err;
                     sa.num_sms = ctx->num_sms;
+                    // a step whose data stay in L2 takes tens of microseconds: its launch latency shows
+                    sa.dep = (double)nb * g.Vs * (3.0 * wfmt_bytes(fmt) + 2.0 * VBY * rn) < 120e6;
                     sa.vstride_in = sa.vstride_out = vsg;
                     for (int k = 0; k < 3; ++k) sa.tile[k] = tile[k];
                     const int sub_groups = kern == TLS_KERNEL_SINGLE ? gn : 1;

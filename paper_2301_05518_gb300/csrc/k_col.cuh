@@ -148,6 +148,8 @@ __global__ void __launch_bounds__(kColMaxThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    grid_dep_launch();
+    grid_dep_wait();
     auto skip = [&](const ColTile &t) {  // serving: no active slot in the group
         if constexpr (ACT) {
             for (int v = 0; v < p.nvg; ++v)
@@ -418,9 +420,8 @@ template <int VP, int WF> cudaError_t col_launch(const StepArgs &a)
             !col_map(mh, a.W, a.g, a.nblk, wfmt_bytes(WF), a.g.hx))
             return cudaErrorNotSupported;
         const int grid = std::min(p.ntile, a.num_sms * occ);
-        kern<<<grid, p.threads + 32, p.smem, a.stream>>>(a.W, a.in, a.out, a.alphaf, a.active, a.g, p, gstride, a.err,
-                                                         mw, mh);
-        return cudaGetLastError();
+        return launch_dep(a.dep, kern, dim3(grid), dim3(p.threads + 32), p.smem, a.stream, a.W, a.in, a.out, a.alphaf,
+                          a.active, a.g, p, gstride, a.err, mw, mh);
     }
 }
 

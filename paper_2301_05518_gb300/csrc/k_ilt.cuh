@@ -40,6 +40,7 @@
 // more (bounded) for its own copies in flight and returns without writing.
 #pragma once
 
+#include "launch.cuh"
 #include "tls_dev.cuh"
 #include "tls_internal.h"
 #include "tma.cuh"
@@ -589,7 +590,10 @@ __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict_
         bool any = false;
 #pragma unroll
         for (int v = 0; v < VB; ++v) any = any || active[il_vec<VP, VB>(t, nvec / VB, v)] != 0;
-        if (!__syncthreads_or(any)) return;
+        if (!__syncthreads_or(any)) {
+            grid_dep_wait();
+            return;
+        }
     }
     // Only the leader touches the mbarrier (initialises it, issues the copies
     // and waits), so no CTA barrier is needed before the copies start.
@@ -599,6 +603,12 @@ __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict_
     }
     constexpr int VBY = vfmt_bytes(VP);
     char *rbuf = ws + 5 * g.hx * wfmt_bytes(WF);
+    if constexpr (!RB) {
+        // W does not change between steps: its copies start before the step before has finished
+        if (leader) ilt_issue_w<WF>(ws, W, g, blk, zq, yq, bar);
+    }
+    grid_dep_launch();
+    grid_dep_wait();
     if (leader) {
         if constexpr (RB) {  // the row's records: its bytes join the phase before the W arrival
             const unsigned rowB = (unsigned)(g.hx * nvec * VBY);
@@ -612,8 +622,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict_
             } else {
                 bulk_load(rbuf, rb + row * nvec * VBY, rowB, bar);
             }
+            ilt_issue_w<WF>(ws, W, g, blk, zq, yq, bar);
         }
-        ilt_issue_w<WF>(ws, W, g, blk, zq, yq, bar);
         if (pfd > 0 && blockIdx.x == 0) ilt_prefetch_ahead<VP, WF>(W, in, g, nvec, pfd);
     }
 
@@ -682,42 +692,23 @@ template <int VP, int WF, int VB> cudaError_t ilt_launch(const StepArgs &a)
                 (int64_t)a.g.hy * a.g.hx * ((int64_t)a.nvec * vfmt_bytes(VP) + 3 * wfmt_bytes(WF));
             pfd = (int)std::max<int64_t>(1, std::min<int64_t>(1 << 16, (int64_t(12) << 20) / plane));
         }
+        auto go = [&](auto kern, auto kern_act, int sm) {
+            return launch_dep(a.dep, act ? kern_act : kern, grid, block, sm, a.stream, a.W, a.in, a.out, a.alphaf, a.active,
+                              a.g, a.nvec, a.err, pfd);
+        };
         if constexpr (VB % 2 == 0) {
             // tile[1] = 8: the row's own records staged with the W rows (one vector group per row)
             const int smem_rb = smem + a.g.hx * a.nvec * vfmt_bytes(VP);
-            if (a.tile[1] == 8 && nvg == a.nvec && smem_rb <= (48 << 10)) {
-                if (act)
-                    k_step_ilt<VP, WF, VB, true, 256, 3, false, true><<<grid, block, smem_rb, a.stream>>>(
-                        a.W, a.in, a.out, a.alphaf, a.active, a.g, a.nvec, a.err, pfd);
-                else
-                    k_step_ilt<VP, WF, VB, false, 256, 3, false, true><<<grid, block, smem_rb, a.stream>>>(
-                        a.W, a.in, a.out, a.alphaf, nullptr, a.g, a.nvec, a.err, pfd);
-                return cudaGetLastError();
-            }
+            if (a.tile[1] == 8 && nvg == a.nvec && smem_rb <= (48 << 10))
+                return go(k_step_ilt<VP, WF, VB, false, 256, 3, false, true>,
+                          k_step_ilt<VP, WF, VB, true, 256, 3, false, true>, smem_rb);
         }
-        if (a.tile[1] == 7 && threads <= 192) {  // registers for 3 CTAs of 192 threads per SM
-            if (act)
-                k_step_ilt<VP, WF, VB, true, 192, 3, true><<<grid, block, smem, a.stream>>>(
-                    a.W, a.in, a.out, a.alphaf, a.active, a.g, a.nvec, a.err, pfd);
-            else
-                k_step_ilt<VP, WF, VB, false, 192, 3, true><<<grid, block, smem, a.stream>>>(
-                    a.W, a.in, a.out, a.alphaf, nullptr, a.g, a.nvec, a.err, pfd);
-        } else if (a.tile[1] == 7) {  // registers for 2 CTAs of 256 threads per SM
-            if (act)
-                k_step_ilt<VP, WF, VB, true, 256, 2, true><<<grid, block, smem, a.stream>>>(
-                    a.W, a.in, a.out, a.alphaf, a.active, a.g, a.nvec, a.err, pfd);
-            else
-                k_step_ilt<VP, WF, VB, false, 256, 2, true><<<grid, block, smem, a.stream>>>(
-                    a.W, a.in, a.out, a.alphaf, nullptr, a.g, a.nvec, a.err, pfd);
-        } else {  // registers for 3 CTAs of 256 threads per SM
-            if (act)
-                k_step_ilt<VP, WF, VB, true, 256, 3><<<grid, block, smem, a.stream>>>(
-                    a.W, a.in, a.out, a.alphaf, a.active, a.g, a.nvec, a.err, pfd);
-            else
-                k_step_ilt<VP, WF, VB, false, 256, 3><<<grid, block, smem, a.stream>>>(
-                    a.W, a.in, a.out, a.alphaf, nullptr, a.g, a.nvec, a.err, pfd);
-        }
-        return cudaGetLastError();
+        if (a.tile[1] == 7 && threads <= 192)  // registers for 3 CTAs of 192 threads per SM
+            return go(k_step_ilt<VP, WF, VB, false, 192, 3, true>, k_step_ilt<VP, WF, VB, true, 192, 3, true>, smem);
+        if (a.tile[1] == 7)  // registers for 2 CTAs of 256 threads per SM
+            return go(k_step_ilt<VP, WF, VB, false, 256, 2, true>, k_step_ilt<VP, WF, VB, true, 256, 2, true>, smem);
+        // registers for 3 CTAs of 256 threads per SM
+        return go(k_step_ilt<VP, WF, VB, false, 256, 3>, k_step_ilt<VP, WF, VB, true, 256, 3>, smem);
     }
 }
 

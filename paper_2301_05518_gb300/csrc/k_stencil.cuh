@@ -121,6 +121,8 @@ __global__ void __launch_bounds__(256) k_step(const char *__restrict__ W, const 
                                               const int *__restrict__ active, SubGeom g, int nblk, int nvec,
                                               int64_t vs_in, int64_t vs_out)
 {
+    grid_dep_launch();
+    grid_dep_wait();
     const int nchunk = (nvec + VB - 1) / VB;
     int64_t site;
     int chunk;
@@ -132,6 +134,62 @@ __global__ void __launch_bounds__(256) k_step(const char *__restrict__ W, const 
     const int64_t boff = (int64_t)blk * g.Ps * VBY;
     site_step<VP, VP, WF, VB, false, false>(W, in, out, alpha, g, blk, i, chunk * VB, nvec, vs_in, vs_out, boff,
                                             boff, active);
+}
+
+// One vector in FP64 on a small lattice: three threads per site, each one row of
+// the result.  The FP64 pipe takes a warp instruction every 16 cycles per SM, so
+// what counts is over how many SMs the warps spread: CTAs of one warp, three times
+// as many as sites / 32.  8^3 (one slice): 12.3 us per step with k_step in CTAs of
+// 128 (4 SMs at work), 4.0 us so.  With more than four warps of sites per SM
+// k_step fills the chip and loads a third of the data.
+template <int WF>
+__global__ void __launch_bounds__(32) k_step_row3(const char *__restrict__ W, const char *__restrict__ in,
+                                                  char *__restrict__ out, const double *__restrict__ alpha, SubGeom g,
+                                                  int nblk)
+{
+    grid_dep_launch();
+    const int row = blockIdx.x % 3;
+    const int site = blockIdx.x / 3 * 32 + threadIdx.x;
+    const bool on = site < nblk * g.Vs;
+    const int blk = on ? site / g.Vs : 0, i = on ? site - blk * g.Vs : 0;
+    constexpr int WB = wfmt_bytes(WF);
+    int fw[3], bw[3];
+    sub_neighbours(g, i, fw, bw);
+    const char *wb = W + (int64_t)blk * 3 * g.Ps * WB;
+    // this row of the forward matrices, this column of the backward ones (W does not change
+    // between steps: loaded before the wait)
+    cpx<double> mf[3][3], mb[3][3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const double2 *p = reinterpret_cast<const double2 *>(wb + d * g.Ps * WB);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double2 f = p[(row * 3 + k) * g.Ps + i], b = p[(k * 3 + row) * g.Ps + bw[d]];
+            mf[d][k] = {f.x, f.y};
+            mb[d][k] = {b.x, b.y};
+        }
+    }
+    grid_dep_wait();
+    if (!on) return;
+    const char *ib = in + (int64_t)blk * g.Ps * vfmt_bytes(P_F64);
+    cpx<double> pf[3][3], pb[3][3], c[3], acc = {0.0, 0.0};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        VFmt<P_F64>::load<false>(ib, g.Ps, fw[d], pf[d]);
+        VFmt<P_F64>::load<false>(ib, g.Ps, bw[d], pb[d]);
+    }
+    VFmt<P_F64>::load<false>(ib, g.Ps, i, c);
+    const cpx<double> cr = row == 0 ? c[0] : row == 1 ? c[1] : c[2];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) cmac(acc, mf[d][k], pf[d][k]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) cmacc(acc, mb[d][k], pb[d][k]);
+    }
+    const double a = alpha[0];
+    double2 *o = reinterpret_cast<double2 *>(out + (int64_t)blk * g.Ps * vfmt_bytes(P_F64));
+    o[row * g.Ps + i] = make_double2(fma(a, fma(-6.0, cr.re, acc.re), cr.re), fma(a, fma(-6.0, cr.im, acc.im), cr.im));
 }
 
 // --------------------------------------------------------------------------
@@ -869,9 +927,15 @@ template <int VP, int WF, int VB> cudaError_t step_launch(const StepArgs &a)
     const int64_t blocks = (items + threads - 1) / threads;
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    k_step<VP, WF, VB><<<(unsigned)blocks, threads, 0, a.stream>>>(a.W, a.in, a.out, a.alpha, a.active, a.g,
-                                                                   a.nblk, a.nvec, a.vstride_in, a.vstride_out);
-    return cudaGetLastError();
+    if constexpr (VP == P_F64 && VB == 1) {
+        if (a.nvec == 1 && !a.active && nsite <= (int64_t)4 * 32 * a.num_sms)
+            return launch_dep(a.dep, k_step_row3<WF>, dim3((unsigned)((nsite + 31) / 32 * 3)), dim3(32), 0, a.stream, a.W,
+                              a.in, a.out, a.alpha, a.g, a.nblk);
+    }
+    // FP64: an early start piles the waiting CTAs on some SMs, whose FP64 pipes then hold up the
+    // step (12^3 x 24: 51 us per step with it, 25 without)
+    return launch_dep(a.dep && VP != P_F64, k_step<VP, WF, VB>, dim3((unsigned)blocks), dim3(threads), 0, a.stream, a.W, a.in, a.out,
+                      a.alpha, a.active, a.g, a.nblk, a.nvec, a.vstride_in, a.vstride_out);
 }
 
 // --------------------------------------------------------------------------

@@ -31,6 +31,7 @@ struct StepArgs {
     int tile[3];           // interleaved kernel: sites per CTA along x', y', z' (0 = a strip along x')
     int *err;              // device error word (kernels with bounded waits); nullable for the others
     int num_sms;           // of the device (persistent CTAs of the column kernel)
+    bool dep;              // short steps: start while the step before drains (launch.cuh)
     cudaStream_t stream;
 };
 
