@@ -917,17 +917,14 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         for (int g0 = 0; g0 < nvec && e == cudaSuccess; g0 += G) {
             const int gn = std::min(G, nvec - g0);
             const int rn = packed_of(gn);
-            const int sub = col ? cp.nvg : gn;  // vectors per interleaved field
             const char *src_g = src_io + (size_t)g0 * io_vec_bytes;
             char *dst_g = dst_io + (size_t)g0 * io_vec_bytes;
             const bool il = il_layout;
             const int m0 = ev_rec(st);
-            if (il) {
-                for (int v = 0; v < gn && e == cudaSuccess; v += sub)
-                    e = launch_pack_il(src_g + (size_t)v * io_vec_bytes, io_prec, vsites,
-                                       (char *)ctx->A.p + (size_t)v * vsg, storage, g, gg->L, t_rel0, ns,
-                                       std::min(sub, gn - v), col ? sub : rn, 0, st, col);
-            } else
+            if (il)
+                e = launch_pack_il(src_g, io_prec, vsites, (char *)ctx->A.p, storage, g, gg->L, t_rel0, ns, gn,
+                                   col ? cp.nvg : rn, 0, st, col);
+            else
                 e = launch_pack_vectors(src_g, io_prec, vsites, (char *)ctx->A.p, storage, vsg, g, gg->L, t_rel0, ns,
                                          gn, st);
             ++launches;
@@ -1002,13 +999,11 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
             }
             const int m2 = ev_rec(st);
             if (e == cudaSuccess) {
-                if (il) {
-                    for (int v = 0; v < gn && e == cudaSuccess; v += sub)
-                        e = launch_unpack_il(result + (size_t)v * vsg, storage, dst_g + (size_t)v * io_vec_bytes, io_prec,
-                                             vsites, g, gg->L, t_rel0, ns, std::min(sub, gn - v), col ? sub : rn, 0, st, col);
-                } else
-                    e = launch_unpack_vectors(result, storage, vsg, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn,
-                                               nullptr, nullptr, st);
+                if (il)
+                    e = launch_unpack_il(result, storage, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn,
+                                         col ? cp.nvg : rn, 0, st, col);
+                else
+                    e = launch_unpack_vectors(result, storage, vsg, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn, st);
                 ++launches;
             }
             const int m3 = ev_rec(st);

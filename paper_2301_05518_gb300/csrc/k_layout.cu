@@ -11,6 +11,7 @@
 // Packed U layout: block b = t * 8 + sub, direction d, entry k = 0..8:
 //   Up[((b * 3 + d) * 9 + k) * Ps + i]  (double2 = one complex entry)
 #include <algorithm>
+#include <type_traits>
 
 #include "tls_dev.cuh"
 #include "tls_internal.h"
@@ -37,28 +38,36 @@ __device__ __forceinline__ Coords coords_of(const SubGeom &g, int sub, int i)
     return c;
 }
 
-// Thread per (canonical site, direction, complex entry), entry fastest: a warp
-// reads 512 contiguous bytes of the canonical links (host memory over C2C
-// included) and scatters them into the 9 planes of each (block, direction).
-__global__ void k_ingest_gauge(const double *__restrict__ U, int nd, double2 *__restrict__ Up, SubGeom g, int Lx,
-                               int Ly, int Lz, int64_t total)
+// CTA = a run of up to kIngestSites sites of one canonical x-row.  The links come in entry by entry
+// (27 consecutive complex numbers a site, coalesced; host memory over C2C included), go through
+// shared memory and leave plane by plane, the even sites of the run and then the odd ones, so that
+// a plane is written in runs of 16-byte words instead of one word per site and plane.  HBM-bound:
+// tls_load_gauge at 48^3 x 64 (device links, 0.15 ms of it cudaMalloc) 2.1 ms before, 1.6
+// now.
+constexpr int kIngestSites = 64;
+__global__ void __launch_bounds__(256) k_ingest_gauge(const double *__restrict__ U, int nd, double2 *__restrict__ Up,
+                                                      SubGeom g, int Lx, int Ly, int Lz, int runs)
 {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
-    const int k = (int)(idx % 27);
-    const int64_t site = idx / 27;
-    const int d = k / 9, e = k - d * 9;
-    const int x = (int)(site % Lx);
-    const int64_t r1 = site / Lx;
-    const int y = (int)(r1 % Ly);
-    const int64_t r2 = r1 / Ly;
-    const int z = (int)(r2 % Lz);
-    const int t = (int)(r2 / Lz);
-    const int sub = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
-    const int i = ((z >> 1) * g.hy + (y >> 1)) * g.hx + (x >> 1);
-    const int b = t * 8 + sub;
-    const double2 v = reinterpret_cast<const double2 *>(U)[(site * nd + d) * 9 + e];
-    Up[(((int64_t)b * 3 + d) * 9 + e) * g.Ps + i] = v;
+    __shared__ double2 sm[27][kIngestSites + 1];
+    const int64_t row = blockIdx.x / runs;  // (t, z, y)
+    const int x0 = (int)(blockIdx.x - row * runs) * kIngestSites;
+    const int n = min(kIngestSites, Lx - x0), h = n / 2;  // x0 and n are even
+    const int y = (int)(row % Ly);
+    const int64_t r2 = row / Ly;
+    const int z = (int)(r2 % Lz), t = (int)(r2 / Lz);
+    const double2 *src = reinterpret_cast<const double2 *>(U) + (row * Lx + x0) * nd * 9;
+    for (int k = threadIdx.x; k < n * 27; k += blockDim.x) {
+        const int x = k / 27, e = k - x * 27;
+        sm[e][(x & 1) * h + (x >> 1)] = src[(int64_t)x * nd * 9 + e];
+    }
+    __syncthreads();
+    const int sub = ((y & 1) << 1) | ((z & 1) << 2);
+    const int i0 = ((z >> 1) * g.hy + (y >> 1)) * g.hx + x0 / 2;
+    for (int k = threadIdx.x; k < n * 27; k += blockDim.x) {
+        const int e = k / n, pos = k - e * n;
+        const int par = pos >= h;
+        Up[((int64_t)(t * 8 + (sub | par)) * 27 + e) * g.Ps + i0 + pos - par * h] = sm[e][pos];
+    }
 }
 
 __global__ void k_export_gauge(const double2 *__restrict__ Up, double *__restrict__ out, SubGeom g, int Lx, int Ly,
@@ -315,66 +324,80 @@ __global__ void k_export_twolink(const char *__restrict__ W, double *__restrict_
     }
 }
 
-template <typename IO, int VP>
-__global__ void k_pack(const IO *__restrict__ src, int64_t svs, char *__restrict__ dst, int64_t dvs, SubGeom g,
-                       int Lx, int Ly, int Lz, int t_first, int64_t nsite)
+// Planar vectors (one vector per launch, persistent forms).  A thread moves the two
+// sites x = 2 x', 2 x' + 1 of a canonical row: 48 (FP64: 96) contiguous bytes of the
+// caller's vector against one site in each of two sublattice blocks, where consecutive
+// lanes are consecutive sites.  HBM-bound; 48^3 x 64, one vector: pack 0.062 ms, unpack
+// 0.160 ms with a thread per site (whose 24-byte pieces lie 48 bytes apart), 0.055 and 0.053 now.
+// AL: the caller's vectors are 16-byte aligned.
+template <typename IO, int VP, bool PACK, bool AL>
+__global__ void __launch_bounds__(256) k_move_planar(std::conditional_t<PACK, const IO, IO> *__restrict__ canon, int64_t cvs,
+                                                     std::conditional_t<PACK, char, const char> *__restrict__ packed,
+                                                     int64_t pvs, SubGeom g, int Ly, int Lz, int t_first, int64_t total)
 {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsite) return;
-    const int v = blockIdx.y;
-    const int b = (int)(s / g.Vs);
-    const int i = (int)(s - (int64_t)b * g.Vs);
-    const int t = t_first + (b >> 3), sub = b & 7;
-    Coords c = coords_of(g, sub, i);
-    const int64_t site = (((int64_t)t * Lz + c.z) * Ly + c.y) * Lx + c.x;
-    const IO *p = src + ((int64_t)v * svs + site) * 6;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= total) return;
+    const int xq = (int)(idx % g.hx);
+    const int64_t row = idx / g.hx;
+    const int y = (int)(row % Ly);
+    const int64_t r2 = row / Ly;
+    const int z = (int)(r2 % Lz), ts = (int)(r2 / Lz);
+    const int sub0 = ((y & 1) << 1) | ((z & 1) << 2);
+    const int i = ((z >> 1) * g.hy + (y >> 1)) * g.hx + xq;
+    auto *p = canon + ((int64_t)blockIdx.y * cvs + ((int64_t)t_first * Lz * Ly + row) * (2 * g.hx) + 2 * xq) * 6;
+    auto *s = packed + (int64_t)blockIdx.y * pvs + (int64_t)(ts * 8 + sub0) * g.Ps * vfmt_bytes(VP);
     typedef typename VFmt<VP>::R R;
-    cpx<R> val[3];
+    constexpr int NV = 16 / sizeof(IO);  // reals per 16-byte word
+    union {
+        float4 q4[3];
+        IO v[12];
+    } w4;
+    IO v[12];
+    if constexpr (PACK) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        val[k].re = (R)p[2 * k];
-        val[k].im = (R)p[2 * k + 1];
-    }
-    VFmt<VP>::template store<false>(dst + (int64_t)v * dvs + (int64_t)b * g.Ps * vfmt_bytes(VP), g.Ps, i, val);
-}
-
-template <typename IO, int VP>
-__global__ void __launch_bounds__(256) k_unpack(const char *__restrict__ src, int64_t svs, IO *__restrict__ dst,
-                                                int64_t dvs, SubGeom g, int Lx, int Ly, int Lz, int t_first,
-                                                int64_t nsite, double *__restrict__ partials)
-{
-    __shared__ double red[256 / 32];
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int v = blockIdx.y;
-    double n2 = 0.0;
-    if (s < nsite) {
-        const int b = (int)(s / g.Vs);
-        const int i = (int)(s - (int64_t)b * g.Vs);
-        const int t = t_first + (b >> 3), sub = b & 7;
-        Coords c = coords_of(g, sub, i);
-        const int64_t site = (((int64_t)t * Lz + c.z) * Ly + c.y) * Lx + c.x;
-        typedef typename VFmt<VP>::R R;
-        cpx<R> val[3];
-        VFmt<VP>::template load<false>(src + (int64_t)v * svs + (int64_t)b * g.Ps * vfmt_bytes(VP), g.Ps, i, val);
-        IO *p = dst + ((int64_t)v * dvs + site) * 6;
+        for (int k = 0; k < 12; k += NV) {
+            if constexpr (AL) {
+                w4.q4[0] = *reinterpret_cast<const float4 *>(p + k);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const IO re = (IO)val[k].re, im = (IO)val[k].im;
-            p[2 * k] = re;
-            p[2 * k + 1] = im;
-            n2 = fma((double)re, (double)re, n2);
-            n2 = fma((double)im, (double)im, n2);
+                for (int j = 0; j < NV; ++j) v[k + j] = w4.v[j];
+            } else {
+#pragma unroll
+                for (int j = 0; j < NV; ++j) v[k + j] = p[k + j];
+            }
         }
     }
-    if (partials == nullptr) return;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) n2 += __shfl_down_sync(0xffffffffu, n2, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = n2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        partials[(int64_t)v * gridDim.x + blockIdx.x] = tot;
+    for (int par = 0; par < 2; ++par) {
+        cpx<R> c[3];
+        auto *blk = s + (int64_t)par * g.Ps * vfmt_bytes(VP);
+        if constexpr (PACK) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                c[k].re = (R)v[6 * par + 2 * k];
+                c[k].im = (R)v[6 * par + 2 * k + 1];
+            }
+            VFmt<VP>::template store<false>(blk, g.Ps, i, c);
+        } else {
+            VFmt<VP>::template load<false>(blk, g.Ps, i, c);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                v[6 * par + 2 * k] = (IO)c[k].re;
+                v[6 * par + 2 * k + 1] = (IO)c[k].im;
+            }
+        }
+    }
+    if constexpr (!PACK) {
+#pragma unroll
+        for (int k = 0; k < 12; k += NV) {
+            if constexpr (AL) {
+#pragma unroll
+                for (int j = 0; j < NV; ++j) w4.v[j] = v[k + j];
+                *reinterpret_cast<float4 *>(p + k) = w4.q4[0];
+            } else {
+#pragma unroll
+                for (int j = 0; j < NV; ++j) p[k + j] = v[k + j];
+            }
+        }
     }
 }
 
@@ -395,19 +418,10 @@ __global__ void __launch_bounds__(256) k_reduce_norms(const double *__restrict__
     if (threadIdx.x == 0) norms[v] = red[0];
 }
 
-// Site i of an interleaved block, in units of rec_n * SB bytes: the colour
-// planes of the block, or (rc) of each x'-row, one row behind the other.
-template <int VP> __device__ __forceinline__ int64_t il_site(const SubGeom &g, int i, bool rc)
-{
-    if (!rc || !il_planes(VP)) return i;
-    const int row = i / g.hx;
-    return (int64_t)row * 2 * g.hx + i;
-}
-
-// Interleaved layout: CTA = (nvec, spb); threadIdx.x = vector, threadIdx.y = site.
+// FP64 records: CTA = (nvec, spb); threadIdx.x = vector, threadIdx.y = site.
 template <typename IO, int VP>
 __global__ void k_pack_il(const IO *__restrict__ src, int64_t svs, char *__restrict__ dst, SubGeom g, int Lx, int Ly,
-                          int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0, bool rc)
+                          int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     if (s >= nsite) return;
@@ -425,13 +439,13 @@ __global__ void k_pack_il(const IO *__restrict__ src, int64_t svs, char *__restr
         val[k].re = (R)p[2 * k];
         val[k].im = (R)p[2 * k + 1];
     }
-    VRec<VP>::store(dst + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + il_site<VP>(g, i, rc) * rec_n * VRec<VP>::SB,
-                    (rc ? g.hx : g.Ps) * rec_n, rec_v0 + v, val);
+    VRec<VP>::store(dst + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + (int64_t)i * rec_n * VRec<VP>::SB, g.Ps * rec_n,
+                    rec_v0 + v, val);
 }
 
 template <typename IO, int VP>
 __global__ void k_unpack_il(const char *__restrict__ src, IO *__restrict__ dst, int64_t dvs, SubGeom g, int Lx,
-                            int Ly, int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0, bool rc)
+                            int Ly, int Lz, int t_first, int64_t nsite, int rec_n, int rec_v0)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     if (s >= nsite) return;
@@ -443,8 +457,8 @@ __global__ void k_unpack_il(const char *__restrict__ src, IO *__restrict__ dst, 
     const int64_t site = (((int64_t)t * Lz + c.z) * Ly + c.y) * Lx + c.x;
     typedef typename VRec<VP>::R R;
     cpx<R> val[3];
-    VRec<VP>::load(src + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + il_site<VP>(g, i, rc) * rec_n * VRec<VP>::SB,
-                   (rc ? g.hx : g.Ps) * rec_n, rec_v0 + v, val);
+    VRec<VP>::load(src + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP) + (int64_t)i * rec_n * VRec<VP>::SB, g.Ps * rec_n,
+                   rec_v0 + v, val);
     IO *p = dst + ((int64_t)v * dvs + site) * 6;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -488,13 +502,12 @@ __global__ void __launch_bounds__(256) k_norm_partials(const IO *__restrict__ ba
 // thread and step.  to_smem selects the direction.
 template <int VP>
 __device__ __forceinline__ void row_copy(unsigned char *smr, const void *gbase, int b, int r, const SubGeom &g, int hx,
-                                         int rec_n, bool to_smem, bool rc)
+                                         int rec_n, bool to_smem)
 {
     constexpr int SB = VRec<VP>::SB;
-    const int nseg = il_planes(VP) && !rc ? 3 : 1;
-    const int segB = hx * rec_n * vfmt_bytes(VP) / nseg;  // one colour, or the whole row
+    const int segB = hx * rec_n * SB;  // one colour (or the whole row for 16-bit records)
+    const int nseg = il_planes(VP) ? 3 : 1;
     char *blk = (char *)gbase + (int64_t)b * g.Ps * rec_n * vfmt_bytes(VP);
-    if (rc) blk += (int64_t)r * rec_n * (vfmt_bytes(VP) - SB);
     for (int c = 0; c < nseg; ++c) {
         uint4 *gs = reinterpret_cast<uint4 *>(blk + ((int64_t)c * g.Ps + r) * rec_n * SB);
         uint4 *ss = reinterpret_cast<uint4 *>(smr + c * segB);
@@ -514,7 +527,7 @@ __device__ __forceinline__ void row_copy(unsigned char *smr, const void *gbase, 
 template <typename IO, int VP>
 __global__ void __launch_bounds__(256) k_unpack_rows(const char *__restrict__ src, IO *__restrict__ dst, int64_t dvs,
                                                      SubGeom g, int Lx, int Ly, int Lz, int t_first, int nvec,
-                                                     int rec_n, int rec_v0, bool rc)
+                                                     int rec_n, int rec_v0)
 {
     extern __shared__ __align__(16) unsigned char smr[];
     constexpr int VBY = vfmt_bytes(VP);
@@ -525,7 +538,7 @@ __global__ void __launch_bounds__(256) k_unpack_rows(const char *__restrict__ sr
     const int r = ((z >> 1) * g.hy + (y >> 1)) * hx;
     const int segB = hx * rec_n * VBY;
     // stage both x'-rows (all rec_n records) with 16-byte loads
-    for (int par = 0; par < 2; ++par) row_copy<VP>(smr + par * segB, src, ts * 8 + (sub0 | par), r, g, hx, rec_n, true, rc);
+    for (int par = 0; par < 2; ++par) row_copy<VP>(smr + par * segB, src, ts * 8 + (sub0 | par), r, g, hx, rec_n, true);
     __syncthreads();
     typedef typename VRec<VP>::R R;
     const int64_t site0 = (((int64_t)(t_first + ts) * Lz + z) * Ly + y) * Lx;
@@ -546,7 +559,7 @@ __global__ void __launch_bounds__(256) k_unpack_rows(const char *__restrict__ sr
 template <typename IO, int VP>
 __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, int64_t svs, char *__restrict__ dst,
                                                    SubGeom g, int Lx, int Ly, int Lz, int t_first, int nvec, int rec_n,
-                                                   int rec_v0, bool rc)
+                                                   int rec_v0)
 {
     extern __shared__ __align__(16) unsigned char smr[];
     constexpr int VBY = vfmt_bytes(VP);
@@ -559,7 +572,7 @@ __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, i
     const bool partial = nvec != rec_n;
     if (partial) {  // keep the records of the other slots: start from the current segments
         for (int par = 0; par < 2; ++par)
-            row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, true, rc);
+            row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, true);
         __syncthreads();
     }
     typedef typename VRec<VP>::R R;
@@ -578,51 +591,185 @@ __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, i
     }
     __syncthreads();
     for (int par = 0; par < 2; ++par)
-        row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, false, rc);
+        row_copy<VP>(smr + par * segB, dst, ts * 8 + (sub0 | par), r, g, hx, rec_n, false);
+}
+
+// --------------------------------------------------------------------------
+// Pack and unpack of the FP32 and 16-bit interleaved records, by vector pairs.
+// A thread moves one record pair of one site: two canonical colour vectors of 24
+// (FP64 caller: 48) bytes each against one 16-byte word per colour, or one 32-byte
+// record.  CTA = one canonical x-row; consecutive lanes take the pairs of a site,
+// then the next site, so that the records of the even and of the odd sites of the
+// row are each written in one contiguous run (nvg = 8: 256 bytes per colour and
+// warp) and the canonical side is read in runs of a few sites per vector, every
+// sector in full.  Both sides go straight between global memory and registers.
+// HBM-bound: 48^3 x 32, 24 vectors, FP32 1.00 / 1.33 ms (pack / unpack) with the
+// rows staged in shared memory one vector at a time, 0.58 / 0.82 now (4.1 GB moved); FP16
+// 2.14 / 1.30, now 0.50 / 0.64.
+// grid.z: vector groups (column kernel), rec_n records each; record rec_v0 + v of a
+// group holds vector v.  A pair of which the caller owns one vector only leaves the
+// other half alone.  AL: the caller's vectors are aligned to a complex number.
+// --------------------------------------------------------------------------
+// Site i of an interleaved block, in units of rec_n * SB bytes: the colour
+// planes of the block, or (rc) of each x'-row, one row behind the other.
+template <int VP> __device__ __forceinline__ int64_t il_site(const SubGeom &g, int i, bool rc)
+{
+    if (!rc || !il_planes(VP)) return i;
+    const int row = i / g.hx;
+    return (int64_t)row * 2 * g.hx + i;
+}
+
+template <typename IO, bool AL> __device__ __forceinline__ void io_load(const IO *p, IO v[6])
+{
+    if constexpr (AL && sizeof(IO) == 4) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float2 q = reinterpret_cast<const float2 *>(p)[c];
+            v[2 * c] = q.x;
+            v[2 * c + 1] = q.y;
+        }
+    } else if constexpr (AL) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 q = reinterpret_cast<const double2 *>(p)[c];
+            v[2 * c] = q.x;
+            v[2 * c + 1] = q.y;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = p[k];
+    }
+}
+
+template <typename IO, bool AL> __device__ __forceinline__ void io_store(IO *p, const cpx<float> x[3])
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if constexpr (AL && sizeof(IO) == 4)
+            reinterpret_cast<float2 *>(p)[c] = make_float2(x[c].re, x[c].im);
+        else if constexpr (AL)
+            reinterpret_cast<double2 *>(p)[c] = make_double2((double)x[c].re, (double)x[c].im);
+        else {
+            p[2 * c] = (IO)x[c].re;
+            p[2 * c + 1] = (IO)x[c].im;
+        }
+    }
+}
+
+struct PairArgs {
+    int64_t vs;            // canonical vector stride in sites
+    int Lx, Ly, Lz, t_first;
+    int nvec, rec_n, rec_v0;
+    int64_t gstride;       // bytes between the fields of two groups
+    bool rc;
+};
+
+template <typename IO, int VP, bool PACK, bool AL>
+__global__ void __launch_bounds__(256) k_move_pairs(std::conditional_t<PACK, const IO, IO> *__restrict__ canon,
+                                                    std::conditional_t<PACK, char, const char> *__restrict__ recs,
+                                                    SubGeom g, PairArgs a)
+{
+    const int y = blockIdx.x % a.Ly, z = blockIdx.x / a.Ly, ts = blockIdx.y;
+    const int first = blockIdx.z * a.rec_n;  // vectors of the groups before this one
+    const int nv = min(a.nvec - first, a.rec_n);
+    const int u0 = a.rec_v0 >> 1, T = ((a.rec_v0 + nv + 1) >> 1) - u0;
+    const int sub0 = ((y & 1) << 1) | ((z & 1) << 2);
+    const int r = ((z >> 1) * g.hy + (y >> 1)) * g.hx;
+    const int64_t site0 = (((int64_t)(a.t_first + ts) * a.Lz + z) * a.Ly + y) * a.Lx;
+    const int64_t sb = (int64_t)a.rec_n * VRec<VP>::SB;
+    const int cs = (int)((a.rc ? g.hx : g.Ps) * a.rec_n);
+    const int64_t row = il_site<VP>(g, r, a.rc);
+    for (int k = threadIdx.x; k < T * a.Lx; k += blockDim.x) {
+        const int x = k / T, u = u0 + k - x * T;
+        const int v0 = 2 * u - a.rec_v0;
+        const bool on0 = v0 >= 0, on1 = v0 + 1 < nv;
+        auto *s = recs + blockIdx.z * a.gstride + ((int64_t)(ts * 8 + (sub0 | (x & 1))) * g.Ps * a.rec_n) * vfmt_bytes(VP) +
+                  (row + (x >> 1)) * sb;
+        auto *p = canon + ((int64_t)(first + v0) * a.vs + site0 + x) * 6;
+        const int64_t next = a.vs * 6;
+        cpx<float> q[2][3];
+        if constexpr (PACK) {
+            IO w[2][6];
+            if (on0) io_load<IO, AL>(p, w[0]);
+            if (on1) io_load<IO, AL>(p + next, w[1]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    q[j][c].re = (float)w[j][2 * c];
+                    q[j][c].im = (float)w[j][2 * c + 1];
+                }
+            if (on0 && on1)
+                VRec<VP>::store2(s, cs, u, q[0], q[1]);
+            else if (on0)
+                VRec<VP>::store(s, cs, 2 * u, q[0]);
+            else
+                VRec<VP>::store(s, cs, 2 * u + 1, q[1]);
+        } else {
+            VRec<VP>::load2(s, cs, u, q[0], q[1]);
+            if (on0) io_store<IO, AL>(p, q[0]);
+            if (on1) io_store<IO, AL>(p + next, q[1]);
+        }
+    }
+}
+
+template <typename IO, bool PACK>
+cudaError_t move_pairs(const void *canon, char *recs, int prec, const SubGeom &g, int nsl, int ngrp, const PairArgs &a,
+                       cudaStream_t s)
+{
+    const dim3 grid((unsigned)(a.Ly * a.Lz), nsl, ngrp);
+    if (nsl > 65535 || ngrp > 65535) return cudaErrorInvalidConfiguration;
+    const bool al = reinterpret_cast<uintptr_t>(canon) % (2 * sizeof(IO)) == 0;
+    auto go = [&](auto k_al, auto k) {
+        if (al)
+            k_al<<<grid, 256, 0, s>>>((IO *)canon, recs, g, a);
+        else
+            k<<<grid, 256, 0, s>>>((IO *)canon, recs, g, a);
+        return cudaGetLastError();
+    };
+    switch (prec) {
+    case P_F32: return go(k_move_pairs<IO, P_F32, PACK, true>, k_move_pairs<IO, P_F32, PACK, false>);
+    case P_F16: return go(k_move_pairs<IO, P_F16, PACK, true>, k_move_pairs<IO, P_F16, PACK, false>);
+    case P_BF16: return go(k_move_pairs<IO, P_BF16, PACK, true>, k_move_pairs<IO, P_BF16, PACK, false>);
+    default: return cudaErrorNotSupported;
+    }
 }
 
 inline int spb_of(int nvec) { return std::max(1, 256 / nvec); }
 
 inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-template <typename IO>
-cudaError_t pack_io(const IO *src, int64_t svs, char *dst, int prec, int64_t dvs, const SubGeom &g, const int L[4],
-                    int t_first, int64_t nsite, int nvec, cudaStream_t s)
+template <typename IO, bool PACK>
+cudaError_t move_planar(const void *canon, int64_t cvs, char *packed, int prec, int64_t pvs, const SubGeom &g,
+                        const int L[4], int t_first, int nsl, int nvec, cudaStream_t s)
 {
-    dim3 grid(nblocks(nsite, 256), nvec);
+    const int64_t total = (int64_t)nsl * L[2] * L[1] * g.hx;
+    const dim3 grid(nblocks(total, 256), nvec);
+    const bool al = reinterpret_cast<uintptr_t>(canon) % 16 == 0;
+    auto go = [&](auto k_al, auto k) {
+        if (al)
+            k_al<<<grid, 256, 0, s>>>((IO *)canon, cvs, packed, pvs, g, L[1], L[2], t_first, total);
+        else
+            k<<<grid, 256, 0, s>>>((IO *)canon, cvs, packed, pvs, g, L[1], L[2], t_first, total);
+        return cudaGetLastError();
+    };
     switch (prec) {
-    case P_F64: k_pack<IO, P_F64><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite); break;
-    case P_F32: k_pack<IO, P_F32><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite); break;
-    case P_F16: k_pack<IO, P_F16><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite); break;
-    case P_BF16: k_pack<IO, P_BF16><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite); break;
+    case P_F64: return go(k_move_planar<IO, P_F64, PACK, true>, k_move_planar<IO, P_F64, PACK, false>);
+    case P_F32: return go(k_move_planar<IO, P_F32, PACK, true>, k_move_planar<IO, P_F32, PACK, false>);
+    case P_F16: return go(k_move_planar<IO, P_F16, PACK, true>, k_move_planar<IO, P_F16, PACK, false>);
+    case P_BF16: return go(k_move_planar<IO, P_BF16, PACK, true>, k_move_planar<IO, P_BF16, PACK, false>);
     default: return cudaErrorNotSupported;
     }
-    return cudaGetLastError();
-}
-
-template <typename IO>
-cudaError_t unpack_io(const char *src, int prec, int64_t svs, IO *dst, int64_t dvs, const SubGeom &g, const int L[4],
-                      int t_first, int64_t nsite, int nvec, double *partials, cudaStream_t s)
-{
-    dim3 grid(nblocks(nsite, 256), nvec);
-    switch (prec) {
-    case P_F64: k_unpack<IO, P_F64><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, partials); break;
-    case P_F32: k_unpack<IO, P_F32><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, partials); break;
-    case P_F16: k_unpack<IO, P_F16><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, partials); break;
-    case P_BF16: k_unpack<IO, P_BF16><<<grid, 256, 0, s>>>(src, svs, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, partials); break;
-    default: return cudaErrorNotSupported;
-    }
-    return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_ingest_gauge(const double *U, int nd, double *Up, const SubGeom &g, const int L[4], cudaStream_t s)
 {
-    const int64_t total = (int64_t)L[0] * L[1] * L[2] * L[3] * 27;
-    if (total == 0) return cudaSuccess;
-    k_ingest_gauge<<<nblocks(total, 256), 256, 0, s>>>(U, nd, reinterpret_cast<double2 *>(Up), g, L[0], L[1], L[2],
-                                                       total);
+    const int runs = (L[0] + kIngestSites - 1) / kIngestSites;
+    const int64_t blocks = (int64_t)L[1] * L[2] * L[3] * runs;
+    if (blocks == 0) return cudaSuccess;
+    k_ingest_gauge<<<(unsigned)blocks, 256, 0, s>>>(U, nd, reinterpret_cast<double2 *>(Up), g, L[0], L[1], L[2], runs);
     return cudaGetLastError();
 }
 
@@ -694,68 +841,28 @@ cudaError_t launch_pack_vectors(const void *src, int io_prec, int64_t src_vstrid
                                 int64_t dst_vstride, const SubGeom &g, const int L[4], int t_first, int nsl,
                                 int nvec, cudaStream_t s)
 {
-    const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
-    if (nsite == 0 || nvec == 0) return cudaSuccess;
+    if ((int64_t)nsl * 8 * g.Vs == 0 || nvec == 0) return cudaSuccess;
     if (io_prec == P_F64)
-        return pack_io<double>((const double *)src, src_vstride_sites, dst, prec, dst_vstride, g, L, t_first, nsite,
-                               nvec, s);
+        return move_planar<double, true>(src, src_vstride_sites, dst, prec, dst_vstride, g, L, t_first, nsl, nvec, s);
     if (io_prec == P_F32)
-        return pack_io<float>((const float *)src, src_vstride_sites, dst, prec, dst_vstride, g, L, t_first, nsite,
-                              nvec, s);
+        return move_planar<float, true>(src, src_vstride_sites, dst, prec, dst_vstride, g, L, t_first, nsl, nvec, s);
     return cudaErrorNotSupported;
 }
-
-int unpack_parts(const SubGeom &g, int nsl) { return (int)nblocks((int64_t)nsl * 8 * g.Vs, 256); }
 
 cudaError_t launch_unpack_vectors(const char *src, int prec, int64_t src_vstride, void *dst, int io_prec,
                                   int64_t dst_vstride_sites, const SubGeom &g, const int L[4], int t_first,
-                                  int nsl, int nvec, double *partials, int *nparts, cudaStream_t s)
+                                  int nsl, int nvec, cudaStream_t s)
 {
-    const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
-    if (nparts) *nparts = unpack_parts(g, nsl);
-    if (nsite == 0 || nvec == 0) return cudaSuccess;
+    if ((int64_t)nsl * 8 * g.Vs == 0 || nvec == 0) return cudaSuccess;
+    char *p = const_cast<char *>(src);
     if (io_prec == P_F64)
-        return unpack_io<double>(src, prec, src_vstride, (double *)dst, dst_vstride_sites, g, L, t_first, nsite,
-                                 nvec, partials, s);
+        return move_planar<double, false>(dst, dst_vstride_sites, p, prec, src_vstride, g, L, t_first, nsl, nvec, s);
     if (io_prec == P_F32)
-        return unpack_io<float>(src, prec, src_vstride, (float *)dst, dst_vstride_sites, g, L, t_first, nsite, nvec,
-                                partials, s);
+        return move_planar<float, false>(dst, dst_vstride_sites, p, prec, src_vstride, g, L, t_first, nsl, nvec, s);
     return cudaErrorNotSupported;
 }
 
-template <typename IO>
-static cudaError_t pack_il_io(const IO *src, int64_t svs, char *dst, int prec, const SubGeom &g, const int L[4],
-                              int t_first, int64_t nsite, int nvec, int rec_n, int rec_v0, bool rc, cudaStream_t s)
-{
-    const int spb = spb_of(nvec);
-    dim3 block(nvec, spb), grid(nblocks(nsite, spb));
-    switch (prec) {
-    case P_F64: k_pack_il<IO, P_F64><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    case P_F32: k_pack_il<IO, P_F32><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    case P_F16: k_pack_il<IO, P_F16><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    case P_BF16: k_pack_il<IO, P_BF16><<<grid, block, 0, s>>>(src, svs, dst, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    default: return cudaErrorNotSupported;
-    }
-    return cudaGetLastError();
-}
-
-template <typename IO>
-static cudaError_t unpack_il_io(const char *src, int prec, IO *dst, int64_t dvs, const SubGeom &g, const int L[4],
-                                int t_first, int64_t nsite, int nvec, int rec_n, int rec_v0, bool rc, cudaStream_t s)
-{
-    const int spb = spb_of(nvec);
-    dim3 block(nvec, spb), grid(nblocks(nsite, spb));
-    switch (prec) {
-    case P_F64: k_unpack_il<IO, P_F64><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    case P_F32: k_unpack_il<IO, P_F32><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    case P_F16: k_unpack_il<IO, P_F16><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    case P_BF16: k_unpack_il<IO, P_BF16><<<grid, block, 0, s>>>(src, dst, dvs, g, L[0], L[1], L[2], t_first, nsite, rec_n, rec_v0, rc); break;
-    default: return cudaErrorNotSupported;
-    }
-    return cudaGetLastError();
-}
-
-bool rows_transpose_ok(const SubGeom &g, int rec_n, int prec, const int L[4])
+static bool rows_transpose_ok(const SubGeom &g, int rec_n, int prec, const int L[4])
 {
     // each colour plane's (or the 16-bit row's) segment is copied in 16-byte words
     const int colB = g.hx * rec_n * il_site_bytes(prec);
@@ -763,74 +870,66 @@ bool rows_transpose_ok(const SubGeom &g, int rec_n, int prec, const int L[4])
     return colB % 16 == 0 && 2 * rowB <= 48 * 1024 && (int64_t)L[1] * L[2] <= 0x7fffffff;
 }
 
+// FP64 records: whole rows through shared memory where they fit, else site by site.
 template <typename IO>
-static cudaError_t rows_io(bool pack, const void *src, int64_t svs, void *dst, int prec, const SubGeom &g,
-                           const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0, bool rc, cudaStream_t s)
+static cudaError_t move_f64(bool pack, const void *canon, int64_t vs, char *recs, const SubGeom &g, const int L[4],
+                            int t_first, int nsl, int nvec, int rec_n, int rec_v0, cudaStream_t s)
 {
-    dim3 grid((unsigned)(L[1] * L[2]), nsl);
-    const int smem = 2 * g.hx * rec_n * vfmt_bytes(prec);
-#define TLS_ROWS_CASE(P)                                                                                            \
-    case P:                                                                                                         \
-        if (pack)                                                                                                   \
-            k_pack_rows<IO, P><<<grid, 256, smem, s>>>((const IO *)src, svs, (char *)dst, g, L[0], L[1], L[2],       \
-                                                      t_first, nvec, rec_n, rec_v0, rc);                                \
-        else                                                                                                        \
-            k_unpack_rows<IO, P><<<grid, 256, smem, s>>>((const char *)src, (IO *)dst, svs, g, L[0], L[1], L[2],     \
-                                                        t_first, nvec, rec_n, rec_v0, rc);                              \
-        break;
-    switch (prec) {
-        TLS_ROWS_CASE(P_F64)
-        TLS_ROWS_CASE(P_F32)
-        TLS_ROWS_CASE(P_F16)
-        TLS_ROWS_CASE(P_BF16)
-    default: return cudaErrorNotSupported;
+    if (rows_transpose_ok(g, rec_n, P_F64, L)) {
+        const dim3 grid((unsigned)(L[1] * L[2]), nsl);
+        const int smem = 2 * g.hx * rec_n * vfmt_bytes(P_F64);
+        if (pack)
+            k_pack_rows<IO, P_F64><<<grid, 256, smem, s>>>((const IO *)canon, vs, recs, g, L[0], L[1], L[2], t_first, nvec,
+                                                          rec_n, rec_v0);
+        else
+            k_unpack_rows<IO, P_F64><<<grid, 256, smem, s>>>(recs, (IO *)canon, vs, g, L[0], L[1], L[2], t_first, nvec,
+                                                            rec_n, rec_v0);
+        return cudaGetLastError();
     }
-#undef TLS_ROWS_CASE
+    const int spb = spb_of(nvec);
+    const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
+    const dim3 block(nvec, spb), grid(nblocks(nsite, spb));
+    if (pack)
+        k_pack_il<IO, P_F64><<<grid, block, 0, s>>>((const IO *)canon, vs, recs, g, L[0], L[1], L[2], t_first, nsite, rec_n,
+                                                    rec_v0);
+    else
+        k_unpack_il<IO, P_F64><<<grid, block, 0, s>>>(recs, (IO *)canon, vs, g, L[0], L[1], L[2], t_first, nsite, rec_n,
+                                                      rec_v0);
     return cudaGetLastError();
+}
+
+template <bool PACK>
+static cudaError_t move_il(const void *canon, int io_prec, int64_t vs, char *recs, int prec, const SubGeom &g,
+                           const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0, cudaStream_t s, bool rc)
+{
+    if ((int64_t)nsl * 8 * g.Vs == 0 || nvec == 0) return cudaSuccess;
+    const int ngrp = rc && rec_v0 == 0 ? (nvec + rec_n - 1) / rec_n : 1;
+    if (nvec > 256 || rec_v0 < 0 || (ngrp == 1 && rec_v0 + nvec > rec_n)) return cudaErrorInvalidValue;
+    if (io_prec != P_F64 && io_prec != P_F32) return cudaErrorNotSupported;
+    if (prec == P_F64) {
+        if (rc) return cudaErrorNotSupported;
+        return io_prec == P_F64
+                   ? move_f64<double>(PACK, canon, vs, recs, g, L, t_first, nsl, nvec, rec_n, rec_v0, s)
+                   : move_f64<float>(PACK, canon, vs, recs, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
+    }
+    const PairArgs a{vs, L[0], L[1], L[2], t_first, nvec, rec_n, rec_v0, (int64_t)nsl * 8 * g.Ps * rec_n * vfmt_bytes(prec), rc};
+    return io_prec == P_F64 ? move_pairs<double, PACK>(canon, recs, prec, g, nsl, ngrp, a, s)
+                            : move_pairs<float, PACK>(canon, recs, prec, g, nsl, ngrp, a, s);
 }
 
 cudaError_t launch_pack_il(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                            const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
                            cudaStream_t s, bool rc)
 {
-    const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
-    if (nsite == 0 || nvec == 0) return cudaSuccess;
-    if (nvec > 256 || rec_v0 < 0 || rec_v0 + nvec > rec_n) return cudaErrorInvalidValue;
-    if (rows_transpose_ok(g, rec_n, prec, L)) {
-        if (io_prec == P_F64)
-            return rows_io<double>(true, src, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
-        if (io_prec == P_F32)
-            return rows_io<float>(true, src, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
-    }
-    if (io_prec == P_F64)
-        return pack_il_io<double>((const double *)src, src_vstride_sites, dst, prec, g, L, t_first, nsite, nvec, rec_n,
-                                  rec_v0, rc, s);
-    if (io_prec == P_F32)
-        return pack_il_io<float>((const float *)src, src_vstride_sites, dst, prec, g, L, t_first, nsite, nvec, rec_n,
-                                 rec_v0, rc, s);
-    return cudaErrorNotSupported;
+    return move_il<true>(src, io_prec, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s, rc);
 }
 
 cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, int64_t dst_vstride_sites,
                              const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
                              cudaStream_t s, bool rc)
 {
-    const int64_t nsite = (int64_t)nsl * 8 * g.Vs;
-    if (nsite == 0 || nvec == 0) return cudaSuccess;
-    if (nvec > 256 || rec_v0 < 0 || rec_v0 + nvec > rec_n) return cudaErrorInvalidValue;
-    if (rows_transpose_ok(g, rec_n, prec, L)) {
-        if (io_prec == P_F64)
-            return rows_io<double>(false, src, dst_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
-        if (io_prec == P_F32)
-            return rows_io<float>(false, src, dst_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, rc, s);
-    }
-    if (io_prec == P_F64)
-        return unpack_il_io<double>(src, prec, (double *)dst, dst_vstride_sites, g, L, t_first, nsite, nvec, rec_n,
-                                    rec_v0, rc, s);
-    if (io_prec == P_F32)
-        return unpack_il_io<float>(src, prec, (float *)dst, dst_vstride_sites, g, L, t_first, nsite, nvec, rec_n,
-                                   rec_v0, rc, s);
-    return cudaErrorNotSupported;
+    return move_il<false>(dst, io_prec, dst_vstride_sites, const_cast<char *>(src), prec, g, L, t_first, nsl, nvec, rec_n,
+                          rec_v0, s, rc);
 }
 
 cudaError_t launch_norm_partials(const void *base, int io_prec, int64_t vstride_sites, int64_t slice_sites, int nsl,

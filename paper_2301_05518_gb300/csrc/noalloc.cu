@@ -183,8 +183,7 @@ extern "C" tls_status tls_smear_noalloc(tls_ctx *ctx, tls_gauge_id id, void *vec
         result = B;
     }
     if (e == cudaSuccess)
-        e = launch_unpack_vectors(result, storage, vs, vecs, io_prec, V, g, gg.L, t_first, nsl, nvec, nullptr, nullptr,
-                                  st);
+        e = launch_unpack_vectors(result, storage, vs, vecs, io_prec, V, g, gg.L, t_first, nsl, nvec, st);
     int herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
     cudaError_t es = cudaStreamSynchronize(st);

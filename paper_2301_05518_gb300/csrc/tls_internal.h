@@ -141,11 +141,10 @@ cudaError_t launch_ape_step(const double *U, double *out, const SubGeom &g, int 
                             cudaStream_t s);
 cudaError_t launch_export_twolink(const char *W, int wfmt, double *out, const SubGeom &g, const int L[4],
                                   cudaStream_t s);
-// Whether the interleaved pack/unpack use the row transposes (contiguous canonical rows).
-bool rows_transpose_ok(const SubGeom &g, int rec_n, int prec, const int L[4]);
 // Interleaved layout: rec_n <= 256 records per site, record (block, i, r).  Caller vector v
-// (0 <= v < nvec) goes to / comes from record rec_v0 + v.  rc: the colour planes are
-// those of each x'-row instead of the block's, so that a row is contiguous (column kernel).
+// (0 <= v < nvec) goes to / comes from record rec_v0 + v.  rc (FP32 and 16-bit): the colour
+// planes are those of each x'-row instead of the block's, so that a row is contiguous, and
+// with rec_v0 = 0 the vectors go to successive fields of rec_n each (column kernel).
 cudaError_t launch_pack_il(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                            const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
                            cudaStream_t s, bool rc = false);
@@ -164,11 +163,10 @@ cudaError_t launch_norm_partials(const void *base, int io_prec, int64_t vstride_
 cudaError_t launch_pack_vectors(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                                 int64_t dst_vstride, const SubGeom &g, const int L[4], int t_first, int nsl,
                                 int nvec, cudaStream_t s);
-// Packed storage -> canonical; partials (nullable) gets one FP64 sum of |psi|^2 per (vector, CTA).
+// Packed storage -> canonical.
 cudaError_t launch_unpack_vectors(const char *src, int prec, int64_t src_vstride, void *dst, int io_prec,
                                   int64_t dst_vstride_sites, const SubGeom &g, const int L[4], int t_first,
-                                  int nsl, int nvec, double *partials, int *nparts, cudaStream_t s);
+                                  int nsl, int nvec, cudaStream_t s);
 cudaError_t launch_reduce_norms(const double *partials, int nparts, int nvec, double *norms, cudaStream_t s);
-int unpack_parts(const SubGeom &g, int nsl);
 
 }  // namespace tls
