@@ -25,8 +25,8 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
 {
     // The kernels that won at some measured shape.  Measured and dropped (they
     // never won at any benchmarked shape): the register-capped and W-staged
-    // interleaved variants, explicit strip lengths, eight vectors per thread in
-    // the packed kernel, the TMA row kernel, the z-marching kernel and both
+    // interleaved variants, explicit strip lengths, eight vectors per thread, the
+    // row kernel with the next hop's records requested early, the TMA row kernel, the z-marching kernel and both
     // persistent forms (tls_smear still runs any of them when asked for).
     std::vector<Cand> c;
     if (nvec <= 4) {
@@ -35,9 +35,9 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
     }
     const int G = std::min(nvec, 256);
     if (storage != TLS_F64) {  // the column kernel at the tile shapes its cost model ranks first
-        ColPlan best[4] = {};
-        double us[4];
-        const int n = col_plans(gg.g, nsl * 8, G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms, best, us, 4);
+        ColPlan best[3] = {};
+        double us[3];
+        const int n = col_plans(gg.g, nsl * 8, G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms, best, us, 3);
         for (int k = 0; k < n; ++k) {
             Cand cd{TLS_KERNEL_MRHS, 2, 0, {0, 0, 0}};
             col_tile_of(best[k], cd.tile);
@@ -56,7 +56,6 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
         // whole rows with the W rows staged by TMA: all vectors or half of them per CTA
         c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 6, 0}});
         c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 6, -1}});  // rows ahead requested into L2
-        c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 7, 0}});
         if (vb % 2 == 0) c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 8, 0}});  // the row's records staged too
         // fewer vectors per CTA: smaller CTAs, W staged once per group (each
         // distinct count once)
@@ -69,11 +68,6 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
         }
         // packed FP32 pairs with the W broadcasts staged by the threads (any row length)
         c.push_back({TLS_KERNEL_MRHS, vb, 128, {0, 2, 0}});
-    }
-    if (storage == TLS_F32 && G2 % 8 == 0) {  // eight FP32 vectors per thread, one colour at a time
-        c.push_back({TLS_KERNEL_MRHS, 8, 0, {0, 6, 0}});
-        c.push_back({TLS_KERNEL_MRHS, 8, 0, {0, 7, 0}});
-        c.push_back({TLS_KERNEL_MRHS, 8, 0, {0, 7, -1}});
     }
     return c;
 }
