@@ -483,6 +483,7 @@ __global__ void __launch_bounds__(256) k_norm_partials(const IO *__restrict__ ba
     const IO *p = base + ((int64_t)v * vstride + (int64_t)sl * slice_sites) * 6;
     const int64_t n = slice_sites * 6;
     double acc = 0.0;
+#pragma unroll 8
     for (int64_t k = (int64_t)part * blockDim.x + threadIdx.x; k < n; k += (int64_t)kNormPartsPerSlice * blockDim.x) {
         const double x = (double)p[k];
         acc = fma(x, x, acc);
