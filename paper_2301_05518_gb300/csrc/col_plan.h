@@ -11,6 +11,7 @@
 namespace tls {
 
 constexpr int kColMaxUnits = 6;
+constexpr int kColMaxGroups = 128;   // vector groups: at most 256 vectors in pairs
 constexpr int kColMaxThreads = 512;  // consumers and the producer warp: 16 warps of 128 registers
 
 TLS_HD inline int up16(int n) { return (n + 15) & ~15; }
@@ -68,6 +69,7 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
     if (nvg < 2 || (nvg & 1) || ny < 1 || ny > g.hy || nseg < 1 || nseg > g.hz) return false;
     p.nvg = nvg;
     p.ngrp = (nvec + nvg - 1) / nvg;
+    if (p.ngrp > kColMaxGroups) return false;
     p.nyt = (g.hy + ny - 1) / ny;
     p.ny = (g.hy + p.nyt - 1) / p.nyt;
     p.nseg = nseg;
@@ -79,7 +81,7 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
     p.w = col_w_plan(wb, g.hx, p.ny);
     p.wB = p.w.bytes;
     if (g.hx > 128 || p.w.nb > 8) return false;
-    p.units = (int)((227 * 1024 - 128) / (p.recB + p.wB));
+    p.units = (int)((226 * 1024 - 128) / (p.recB + p.wB));
     if (p.units < 3) return false;
     if (p.units > kColMaxUnits) p.units = kColMaxUnits;
     p.smem = 128 + p.units * (p.recB + p.wB);

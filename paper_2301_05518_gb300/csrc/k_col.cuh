@@ -105,11 +105,12 @@ struct ColTile {
     int grp, blk, z0, n, y0, nyl;
 };
 
-__device__ __forceinline__ ColTile col_tile(int tile, const ColPlan &p, const SubGeom &g)
+// ngrp: vector groups that have tiles (serving: those with an active slot).
+__device__ __forceinline__ ColTile col_tile(int tile, int ngrp, const ColPlan &p, const SubGeom &g)
 {
     ColTile t;
-    t.grp = tile % p.ngrp;
-    int r = tile / p.ngrp;
+    t.grp = tile % ngrp;
+    int r = tile / ngrp;
     const int yt = r % p.nyt;
     r /= p.nyt;
     const int seg = r % p.nseg;
@@ -147,16 +148,34 @@ __global__ void __launch_bounds__(kColMaxThreads, 1)
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // Serving: only the groups with an active slot have tiles, so that the CTAs share them evenly
+    // whatever their number (skipped tile by tile, a stride of 152 CTAs over 4 groups left half the
+    // CTAs without work when two groups were active).
+    __shared__ int act_grp[ACT ? kColMaxGroups + 1 : 1];  // their indices, then their number
+    if constexpr (ACT) {
+        if (tid < 32) {
+            int n = 0;
+            for (int g0 = 0; g0 < p.ngrp; g0 += 32) {
+                const int grp = g0 + lane;
+                bool any = false;
+                if (grp < p.ngrp)
+                    for (int v = 0; v < p.nvg; ++v) any = any || active[grp * p.nvg + v] != 0;
+                const unsigned m = __ballot_sync(0xffffffffu, any);
+                if (any) act_grp[n + __popc(m & ((1u << lane) - 1u))] = grp;
+                n += __popc(m);
+            }
+            if (lane == 0) act_grp[kColMaxGroups] = n;
+        }
+    }
     __syncthreads();
     grid_dep_launch();
     grid_dep_wait();
-    auto skip = [&](const ColTile &t) {  // serving: no active slot in the group
-        if constexpr (ACT) {
-            for (int v = 0; v < p.nvg; ++v)
-                if (active[t.grp * p.nvg + v]) return false;
-            return true;
-        }
-        return false;
+    const int ngrp = ACT ? act_grp[kColMaxGroups * ACT] : p.ngrp;
+    const int ntile = ACT ? p.ntile / p.ngrp * ngrp : p.ntile;
+    auto tile_at = [&](int tile) {
+        ColTile t = col_tile(tile, ngrp, p, g);
+        if constexpr (ACT) t.grp = act_grp[t.grp];
+        return t;
     };
 
     if (tid >= p.threads) {
@@ -188,9 +207,8 @@ __global__ void __launch_bounds__(kColMaxThreads, 1)
         int slot = 0, issued = 0;
         unsigned phase = 1;  // empty[] parity to wait for: the first pass through the ring does not wait
         bool ok = true;
-        for (int tile = blockIdx.x; tile < p.ntile && ok; tile += gridDim.x) {
-            const ColTile t = col_tile(tile, p, g);
-            if (skip(t)) continue;
+        for (int tile = blockIdx.x; tile < ntile && ok; tile += gridDim.x) {
+            const ColTile t = tile_at(tile);
             const int ym = t.y0 == 0 ? hy - 1 : t.y0 - 1;
             const bool up = t.y0 > 0, dn = t.y0 + t.nyl < hy;  // halo rows next to the main rows
             const char *src0 = nullptr;
@@ -294,9 +312,8 @@ __global__ void __launch_bounds__(kColMaxThreads, 1)
             phase ^= 1;
         }
     };
-    for (int tile = blockIdx.x; tile < p.ntile; tile += gridDim.x) {
-        const ColTile t = col_tile(tile, p, g);
-        if (skip(t)) continue;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        const ColTile t = tile_at(tile);
         const bool mine = yl < t.nyl;
         const int v = t.grp * p.nvg + 2 * tp;
         const float2 a2 = *reinterpret_cast<const float2 *>(alphaf + v);
