@@ -296,6 +296,7 @@ typedef struct {
                             /* vectors per group (even), tile[2] = rows per    */
                             /* tile | z segments << 8 | ring units << 16 (a    */
                             /* shape that does not fit goes to the planner);   */
+                            /* 10 keeps planar vectors, up to 8 in one launch; */
                             /* tile[2] (tile[1] = 6..8): each CTA requests     */
                             /* into L2 the W rows and records of the row       */
                             /* tile[2] planes ahead in launch order; 0 none,   */

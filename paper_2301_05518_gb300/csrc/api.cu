@@ -705,7 +705,9 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         auto it = ctx->tune.find(key);
         const bool have = it != ctx->tune.end();
         if (kern == TLS_KERNEL_AUTO) {
-            kern = have ? it->second.kernel : (nvec == 1 ? TLS_KERNEL_SINGLE : TLS_KERNEL_MRHS);
+            kern = have ? it->second.kernel
+                   : nvec == 1 || (storage == TLS_F64 && op == 0 && il_f64_lanes(nvec, g.hx) < 0.97) ? TLS_KERNEL_SINGLE
+                                                                                                    : TLS_KERNEL_MRHS;
         }
         if (have && it->second.kernel == kern) {
             vb = it->second.vb;
@@ -739,7 +741,11 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     if (col_ok && planned) {
         double us = 0;
         const double row_us = row_estimate(g, nblk, col_n, VBY, wfmt_bytes(fmt));
-        if (col_plans(g, nblk, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1) && us < row_us) {
+        const bool have_col = col_plans(g, nblk, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1) > 0;
+        if (planar_ok(g, nblk, nvec, wfmt_bytes(fmt)) &&
+            planar_estimate(g, nblk, nvec, VBY, wfmt_bytes(fmt)) < (have_col ? std::min(us, row_us) : row_us)) {
+            tile[1] = 10;
+        } else if (have_col && us < row_us) {
             col = true;
             col_tile_of(cp, tile);
         } else {
@@ -774,7 +780,13 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         if (threads <= 0) threads = 256;
     }
     // The multi-RHS kernel works on the interleaved layout in groups of <= 256 vectors.
-    const bool il_layout = kern == TLS_KERNEL_MRHS || kern == TLS_KERNEL_MRHS_ROWS || kern == TLS_KERNEL_MRHS_ZM;
+    // tile[1] = 10: planar vectors, all of them in one launch (few vectors)
+    const bool planar = kern == TLS_KERNEL_MRHS && op == 0 && tile[1] == 10 && nvec <= 8;
+    if (planar) {
+        vb = planar_vb(storage, nvec);
+        threads = 128;
+    }
+    const bool il_layout = !planar && (kern == TLS_KERNEL_MRHS || kern == TLS_KERNEL_MRHS_ROWS || kern == TLS_KERNEL_MRHS_ZM);
     const int G = il_layout ? std::min(nvec, 256) : nvec;
 
     // Host vectors go through bulk copies (DMA) into a staging buffer.  On a
@@ -976,6 +988,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
                     for (int k = 0; k < 3; ++k) sa.tile[k] = tile[k];
                     const int sub_groups = kern == TLS_KERNEL_SINGLE ? gn : 1;
                     sa.nvec = kern == TLS_KERNEL_SINGLE ? 1 : rn;
+                    if (planar) sa.nvec = gn;
                     for (int gi = 0; gi < sub_groups && e == cudaSuccess; ++gi) {
                         char *x = (char *)ctx->A.p + (size_t)gi * vsg;
                         char *y = (char *)ctx->B.p + (size_t)gi * vsg;

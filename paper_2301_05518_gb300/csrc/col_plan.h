@@ -125,13 +125,37 @@ inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby
 // us), with the arithmetic of the W formats shared by four vectors (24 vectors at
 // 48^3 x 32, row / column kernel: f32-18 1018 / 927, f32-12 1103 / 1065, f32-8 1699 /
 // above 2600, 16-bit vectors with f32-18 1203 / 1037, with f16-12 1393 / 1414 us).
+// Rows (CTAs of the row kernel): one starts about every nanosecond (16^3 x 32: 16384 of them,
+// 17.7 us per step with 3 vectors).
+inline double row_ctas(const SubGeom &g, int nblk) { return (double)nblk * g.hy * g.hz; }
+
 inline double row_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb)
 {
     const int n = (nvec + 1) & ~1;
     const double fmt = wb == 48 ? 1.08 : wb == 32 ? 1.65 : wb == 24 ? 1.15 : 1.0;
     const double site = n % 4 ? 0.02 + 0.015 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
     const bool tma = (g.hx * (wb % 16)) % 16 == 0;
-    return (double)nblk * g.Vs * site * 1e-3 * (tma ? 1.0 : 1.75) * (vby == 16 ? 1.2 : 1.0) * fmt + 4;
+    const double us = (double)nblk * g.Vs * site * 1e-3 * (tma ? 1.0 : 1.75) * (vby == 16 ? 1.2 : 1.0) * fmt;
+    return std::max(us, row_ctas(g, nblk) * 1e-3) + 2;
+}
+
+// All vectors in one launch of the planar kernel, two or four a thread: reads W once, has
+// no rows to keep whole, but pays for unused lanes of its four vectors (16^3 x 32, 2 / 3 / 4
+// vectors: 7.0 / 11.3 / 13.9 us per step against 12.1 / 17.7 / 17.7; 48^3 x 32: 202 / 375 /
+// 460 against 186 / 231 / 231; 32^3 x 16, 2 FP16 vectors with W f16-12: 27 against 47).
+// A candidate for two vectors, and for up to four where the row kernel is bound by starting
+// its CTAs.  Not for the 8-real W, whose reconstruction rounds differently there.
+inline bool planar_ok(const SubGeom &g, int nblk, int nvec, int wb)
+{
+    return wb != 32 && (nvec == 2 || (nvec > 2 && nvec <= 4 && row_ctas(g, nblk) > 8000));
+}
+
+inline double planar_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb)
+{
+    const double sites = (double)nblk * g.Vs;
+    const double site = nvec == 2 ? 0.06 : nvec == 3 ? 0.108 : 0.132;
+    const double l2 = sites * (3.0 * wb + 2.0 * vby * nvec) < 60e6 ? 0.7 : 1.0;  // stays in L2
+    return sites * site * l2 * (wb == 48 ? 1.15 : 1.0) * (vby == 16 ? 0.9 : 1.0) * 1e-3 + 2.5;
 }
 
 // The best tile shapes by that estimate, best first (at most `most`).  nvg divides
@@ -194,6 +218,34 @@ inline int row_tile(const SubGeom &g, int nblk, int nvec, int vby, int tile[3])
     tile[1] = 6;
     tile[2] = (double)nblk * g.Vs * (216.0 + 2.0 * vby * n) > 120e6 ? -1 : 0;
     return n % 4 == 0 && n / 4 * g.hx >= (vby == 16 ? 64 : 20) ? 4 : 2;
+}
+
+// Vectors per thread of the planar kernel when it takes several at once.
+inline int planar_vb(int storage, int nvec)
+{
+    const int cap = storage == P_F64 ? 4 : 8;
+    int vb = 2;
+    while (vb < cap && vb < nvec) vb *= 2;
+    return vb;
+}
+
+// Share of the lanes of a warp at work in the FP64 multi-RHS kernel (nvec threads per site, a
+// strip of one row per CTA of at most 256 threads).  The FP64 pipe bounds it, so idle lanes cost
+// their share, and one vector per launch, which has none, reads W more often for nothing lost
+// (32^3 x 16, 3 vectors: 48 of 64 lanes, 779 us per step against 597; 4 vectors: 779 against 796).
+inline double il_f64_lanes(int nvec, int hx)
+{
+    const int n = nvec < 256 ? nvec : 256;
+    int spb = std::max(1, 256 / n);
+    for (int s = spb; s >= 1; --s)
+        if ((s * n) % 32 == 0) {
+            spb = s;
+            break;
+        }
+    spb = std::min(spb, hx);
+    const int strips = (hx + spb - 1) / spb;  // the last one may be short, its CTA is not
+    const double threads = (double)strips * ((spb * n + 31) / 32 * 32);
+    return (double)hx * n / threads;
 }
 
 }  // namespace tls

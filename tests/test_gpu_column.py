@@ -64,25 +64,29 @@ def test_column_kernel_bitwise_equals_single(ctx, T, dims, nvec, storage, wprec,
 @pytest.mark.parametrize("dims,nvec,storage", [((16, 16, 16, 8), 3, "F32"), ((30, 18, 22, 4), 7, "F32"),
                                                ((32, 32, 32, 4), 12, "F16"), ((24, 24, 24, 8), 72, "F32"),
                                                ((50, 10, 10, 2), 24, "BF16"), ((8, 8, 4, 2), 301, "F32"),
-                                               ((4, 4, 4, 2), 1, "F32")])
+                                               ((4, 4, 4, 2), 1, "F32"), ((16, 16, 16, 32), 4, "F32"),
+                                               ((10, 6, 8, 3), 2, "F16"), ((6, 6, 10, 2), 3, "F64"),
+                                               ((16, 8, 8, 2), 4, "F64")])
 def test_planner_choice_bitwise_equals_single(ctx, T, dims, nvec, storage):
     """Without a tune entry the planner picks the kernel and the tile shape: same results, host
     buffers included."""
     U = synth.gauge_haar(dims, 53, nd=3)
-    vecs = synth.gaussian_vectors(dims, nvec, 54, dtype=torch.complex64)
+    f64 = storage == "F64"
+    vecs = synth.gaussian_vectors(dims, nvec, 54, dtype=torch.complex128 if f64 else torch.complex64)
     st = getattr(T, "TLS_" + storage)
+    io = T.TLS_F64 if f64 else T.TLS_F32
     gid = ctx.load_gauge(U, 3, dims)
-    ctx.build_twolink(gid, T.TLS_F32, 18)
+    ctx.build_twolink(gid, io, 18)
     for t0 in (-1, 1):
         want = vecs.clone().cuda()
-        nw = ctx.smear(gid, want, T.TLS_F32, nvec, 4, 0.9, timeslice=t0, storage=st, kernel=T.TLS_KERNEL_SINGLE,
+        nw = ctx.smear(gid, want, io, nvec, 4, 0.9, timeslice=t0, storage=st, kernel=T.TLS_KERNEL_SINGLE,
                        norms=True)
         for kern in (T.TLS_KERNEL_AUTO, T.TLS_KERNEL_MRHS):
             got = vecs.clone().cuda()
-            ng = ctx.smear(gid, got, T.TLS_F32, nvec, 4, 0.9, timeslice=t0, storage=st, kernel=kern, norms=True)
+            ng = ctx.smear(gid, got, io, nvec, 4, 0.9, timeslice=t0, storage=st, kernel=kern, norms=True)
             assert torch.equal(got, want) and (ng == nw).all()
         host = vecs.clone()
-        ctx.smear(gid, host, T.TLS_F32, nvec, 4, 0.9, timeslice=t0, storage=st)
+        ctx.smear(gid, host, io, nvec, 4, 0.9, timeslice=t0, storage=st)
         assert torch.equal(host, want.cpu())
     ctx.free_gauge(gid)
 
