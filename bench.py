@@ -94,6 +94,10 @@ def kernel_symbol(kern_name: str, entry: dict) -> str:
     """CUDA kernel that a tune-table entry launches (the name ncu lists)."""
     if kern_name == "mrhs":
         tile = tuple(entry.get("tile", (0, 0, 0)))
+        if tile[1] == 9:
+            return "k_step_col"
+        if tile[1] == 10:
+            return "k_step"
         if tile[1] in (6, 7, 8):
             return "k_step_ilt"
         if tile[1] == 5:

@@ -747,6 +747,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
             tile[1] = 10;
         } else if (have_col && us < row_us) {
             col = true;
+            vb = 2;
             col_tile_of(cp, tile);
         } else {
             vb = row_tile(g, nblk, col_n, VBY, tile);

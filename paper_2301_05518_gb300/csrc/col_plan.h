@@ -11,6 +11,7 @@
 namespace tls {
 
 constexpr int kColMaxUnits = 6;
+constexpr int kColMaxSmem = 226 * 1024;  // of 227 KB, beside the serving form's list of groups
 constexpr int kColMaxGroups = 128;   // vector groups: at most 256 vectors in pairs
 constexpr int kColMaxThreads = 512;  // consumers and the producer warp: 16 warps of 128 registers
 
@@ -81,7 +82,7 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
     p.w = col_w_plan(wb, g.hx, p.ny);
     p.wB = p.w.bytes;
     if (g.hx > 128 || p.w.nb > 8) return false;
-    p.units = (int)((226 * 1024 - 128) / (p.recB + p.wB));
+    p.units = (int)((kColMaxSmem - 128) / (p.recB + p.wB));
     if (p.units < 3) return false;
     if (p.units > kColMaxUnits) p.units = kColMaxUnits;
     p.smem = 128 + p.units * (p.recB + p.wB);
@@ -100,7 +101,8 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
 // scheduler; the copies, 36.5 bytes per cycle; and, with d units in flight, 1/d of
 // a copy's latency of 2350 cycles plus its transfer.  A tile of n planes takes n + 2
 // units; the whole cannot beat the memory.  A thread rebuilds W for one vector pair
-// only, so W formats that need arithmetic cost it more than the row kernel.
+// only, so W formats that need arithmetic cost it more than the row kernel; groups of
+// two or four vectors measured about an eighth above the fit.
 inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby, int wb, int num_sms)
 {
     const int warps = p.threads / 32;
@@ -108,7 +110,7 @@ inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby
     while ((occ + 1) * (warps + 1) <= 16 && (occ + 1) * (p.smem + 1024) <= 228 * 1024) ++occ;
     const int eff = std::min(occ, (p.ntile + num_sms - 1) / num_sms);
     const double rounds = (p.ntile + num_sms * eff - 1) / (num_sms * eff);
-    const double fmt = wb == 72 ? 1.0 : wb == 48 || wb == 36 ? 1.15 : wb == 24 ? 1.4 : 4.0;
+    const double fmt = (wb == 72 ? 1.0 : wb == 48 || wb == 36 ? 1.15 : wb == 24 ? 1.7 : 4.0) * (p.nvg <= 4 ? 1.12 : 1.0);
     const double unit = p.recB + p.wB;
     const double comp = (356 + 650.0 * ((warps * eff + 3) / 4)) * (vby == 16 ? 1.145 : 1.0) * fmt;
     const double copy = eff * unit / 36.5, lat = (2350 + unit / 36.5) / (p.units - 2);

@@ -446,7 +446,8 @@ template <int VP, int WF> cudaError_t col_launch(const StepArgs &a)
         p.smem = 128 + p.units * (p.recB + p.wB);
         const int64_t gstride = (int64_t)a.nblk * a.g.Ps * p.nvg * vfmt_bytes(VP);
         auto kern = a.active ? k_step_col<VP, WF, true> : k_step_col<VP, WF, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+        // always the same value: the attribute belongs to the function, other threads may launch it too
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kColMaxSmem);
         int occ = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, p.threads + 32, p.smem);
         if (e != cudaSuccess) return e;

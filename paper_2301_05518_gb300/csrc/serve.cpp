@@ -75,6 +75,8 @@ struct Batch {
     cudaStream_t stream = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool launched = false;
+    const char *W = nullptr; // two-link field and format the batch was made for (its graphs hold them)
+    int wfmt = -1;
     bool col = false;        // column kernel: slots in groups of cp.nvg, one interleaved field behind the other
     ColPlan cp{};
     int *d_err = nullptr;    // device error word of this batch's kernels (bounded waits)
@@ -149,6 +151,8 @@ tls_status make_batch(tls_ctx *ctx, Server *sv, const BatchKey &key, const Gauge
     b->S = batch_slots(key.storage, sv->opts.max_slots);
     b->K = sv->opts.steps_per_launch;
     b->vb = default_il_vb(key.storage, b->S);
+    b->W = gg.W;
+    b->wfmt = gg.wfmt;
     if (key.storage != TLS_F64) {
         // The column kernel skips slot groups without an active slot (so does the row kernel, by
         // its larger CTA groups); it is taken unless the row kernel is clearly faster with every
@@ -268,6 +272,12 @@ int try_admit(tls_ctx *ctx, Server *sv, Job *j)
     BatchKey key{j->d.gauge, j->d.storage, j->d.timeslice};
     Batch *b = nullptr;
     auto bit = sv->batches.find(key);
+    if (bit != sv->batches.end() && bit->second->used_slots() == 0 &&
+        (bit->second->W != gg.W || bit->second->wfmt != gg.wfmt)) {  // W was rebuilt since
+        destroy_batch(ctx, bit->second.get());
+        sv->batches.erase(bit);
+        bit = sv->batches.end();
+    }
     if (bit != sv->batches.end()) {
         b = bit->second.get();
     } else {

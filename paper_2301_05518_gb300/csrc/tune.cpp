@@ -38,6 +38,8 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
         ColPlan best[3] = {};
         double us[3];
         const int n = col_plans(gg.g, nsl * 8, G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms, best, us, 3);
+        if (nvec >= 2 && nvec <= 4 && gg.wfmt != W_F32_8)  // planar vectors in one launch
+            c.push_back({TLS_KERNEL_MRHS, planar_vb(storage, nvec), 128, {0, 10, 0}});
         for (int k = 0; k < n; ++k) {
             Cand cd{TLS_KERNEL_MRHS, 2, 0, {0, 0, 0}};
             col_tile_of(best[k], cd.tile);

@@ -108,3 +108,21 @@ def test_padded_groups_do_not_cost_admission(T):
         c.smear(gid, one, T.TLS_F32, 1, 3, 0.6, kernel=T.TLS_KERNEL_SINGLE)
         c.smear(gid, x, T.TLS_F32, nvec, 3, 0.6)
         assert torch.equal(x[7:8], one)
+
+
+def test_serving_batch_follows_a_rebuilt_field(T):
+    """An idle batch made for one two-link field is not reused after tls_build_twolink replaced it."""
+    dims = (16, 16, 16, 4)
+    with T.Context(0) as c:
+        gid = c.load_gauge(synth.gauge_haar(dims, 57, nd=3).cuda(), 3, dims)
+        vecs = synth.gaussian_vectors(dims, 5, 58, dtype=torch.complex64)
+        c.build_twolink(gid, T.TLS_F32, 18)
+        c.serve_start(max_slots=12, steps_per_launch=2, use_graphs=1)
+        for recon in (18, 12, 18):
+            c.build_twolink(gid, T.TLS_F32, recon)
+            got, want = vecs.clone().cuda(), vecs.clone().cuda()
+            torch.cuda.synchronize()
+            c.serve_wait(c.serve_submit(gid, got, T.TLS_F32, 5, 7, 1.4), 60)
+            c.smear(gid, want, T.TLS_F32, 5, 7, 1.4, kernel=T.TLS_KERNEL_MRHS)
+            assert torch.equal(got, want)
+        c.serve_stop()
