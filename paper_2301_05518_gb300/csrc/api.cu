@@ -147,17 +147,6 @@ cudaError_t launch_step_il(const StepArgs &a)
     }
 }
 
-cudaError_t launch_hop(const StepArgs &a)
-{
-    switch (a.prec_in) {
-    case P_F64: return launch_hop_f64(a);
-    case P_F32: return launch_hop_f32(a);
-    case P_F16: return launch_hop_f16(a);
-    case P_BF16: return launch_hop_bf16(a);
-    default: return cudaErrorNotSupported;
-    }
-}
-
 cudaError_t launch_step_col(const StepArgs &a)
 {
     switch (a.prec_in) {
@@ -544,7 +533,10 @@ tls_status tls_build_links(tls_ctx *ctx, tls_gauge_id id, int prec, int keep_U, 
     if (fmt < 0) return fail(TLS_ERR_UNSUPPORTED, "tls_build_links: precision %d (TLS_F64 or TLS_F32)", prec);
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t bytes = (size_t)gg->L[3] * 8 * 3 * gg->g.Ps * wfmt_bytes(fmt);
+    // FP32 links: whole slices in canonical order, for the step kernels (slice_geom)
+    const SubGeom gc = slice_geom(gg->L);
+    const bool whole = fmt == W_F32_18;
+    const size_t bytes = (whole ? (size_t)gg->L[3] * 3 * gc.Ps : (size_t)gg->L[3] * 8 * 3 * gg->g.Ps) * wfmt_bytes(fmt);
     if (gg->L1 && gg->L1_bytes != bytes) {
         dev_free(ctx, gg->L1, gg->L1_bytes);
         gg->L1 = nullptr;
@@ -555,7 +547,8 @@ tls_status tls_build_links(tls_ctx *ctx, tls_gauge_id id, int prec, int keep_U, 
         if (s != TLS_OK) return s;
         gg->L1_bytes = bytes;
     }
-    cudaError_t e = launch_build_links(gg->Up, gg->L1, fmt, gg->g, gg->L[3] * 8, st);
+    cudaError_t e = whole ? launch_build_links_slices(gg->Up, gg->L1, gg->g, gc, gg->L[3], st)
+                          : launch_build_links(gg->Up, gg->L1, fmt, gg->g, gg->L[3] * 8, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "tls_build_links");
     gg->l1fmt = fmt;
@@ -683,10 +676,13 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
 
-    const SubGeom &g = gg->g;
+    // The FP32 and 16-bit one-link step works on whole slices: one block per slice.
+    const bool whole = op == 1 && storage != TLS_F64;
+    const SubGeom g = whole ? slice_geom(gg->L) : gg->g;
+    const int bps = whole ? 1 : 8;  // blocks per slice
     const int nsl = timeslice < 0 ? gg->L[3] : 1;
     const int t_first = timeslice < 0 ? 0 : timeslice;
-    const int nblk = nsl * 8;
+    const int nblk = nsl * bps;
     const int64_t Vslice = (int64_t)gg->L[0] * gg->L[1] * gg->L[2];
     const int64_t V = Vslice * gg->L[3];
     const int VBY = vfmt_bytes(storage);
@@ -722,14 +718,15 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         for (int k = 0; k < 3; ++k) tile[k] = force_tile[k];
         planned = false;
     }
-    if (op == 1) {  // one-link hops: the interleaved kernel only
+    if (op == 1) {  // one-link hops: multi-RHS only, the table is for the two-link step
         kern = TLS_KERNEL_MRHS;
+        vb = threads = 0;
         for (int k = 0; k < 3; ++k) tile[k] = 0;
-        planned = false;
+        planned = whole;
     }
     // The column kernel (tile[1] = 9) works on vector groups of tile[0], one interleaved field
     // behind the other; a shape it does not take goes to the planner.
-    const bool col_ok = kern == TLS_KERNEL_MRHS && op == 0 && storage != TLS_F64;
+    const bool col_ok = kern == TLS_KERNEL_MRHS && storage != TLS_F64;
     const int col_n = std::min(nvec, 256);
     ColPlan cp{};
     bool col = false;
@@ -742,7 +739,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         double us = 0;
         const double row_us = row_estimate(g, nblk, col_n, VBY, wfmt_bytes(fmt));
         const bool have_col = col_plans(g, nblk, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1) > 0;
-        if (planar_ok(g, nblk, nvec, wfmt_bytes(fmt)) &&
+        if (op == 0 && planar_ok(g, nblk, nvec, wfmt_bytes(fmt)) &&
             planar_estimate(g, nblk, nvec, VBY, wfmt_bytes(fmt)) < (have_col ? std::min(us, row_us) : row_us)) {
             tile[1] = 10;
         } else if (have_col && us < row_us) {
@@ -923,9 +920,9 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     // the same norms).
     const size_t io_elem_b = io_elem;
     auto run_slices = [&](const char *src_io, char *dst_io, int64_t vsites, int t_rel0, int t_abs, int ns) {
-        const int nb = ns * 8;
+        const int nb = ns * bps;
         const int64_t vsg = (int64_t)nb * g.Ps * VBY;  // packed bytes per vector of these slices
-        const char *Wg = field + (size_t)t_abs * 8 * 3 * g.Ps * wfmt_bytes(fmt);
+        const char *Wg = field + (size_t)t_abs * bps * 3 * g.Ps * wfmt_bytes(fmt);
         const size_t io_vec_bytes = (size_t)vsites * 6 * io_elem_b;
         for (int g0 = 0; g0 < nvec && e == cudaSuccess; g0 += G) {
             const int gn = std::min(G, nvec - g0);
@@ -936,7 +933,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
             const int m0 = ev_rec(st);
             if (il)
                 e = launch_pack_il(src_g, io_prec, vsites, (char *)ctx->A.p, storage, g, gg->L, t_rel0, ns, gn,
-                                   col ? cp.nvg : rn, 0, st, col);
+                                   col ? cp.nvg : rn, 0, st, col, whole);
             else
                 e = launch_pack_vectors(src_g, io_prec, vsites, (char *)ctx->A.p, storage, vsg, g, gg->L, t_rel0, ns,
                                          gn, st);
@@ -983,6 +980,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
                     sa.stream = st;
                     sa.err = ctx->d_err;
                     sa.num_sms = ctx->num_sms;
+                    sa.hop = op == 1;
                     // a step whose data stay in L2 takes tens of microseconds: its launch latency shows
                     sa.dep = (double)nb * g.Vs * (3.0 * wfmt_bytes(fmt) + 2.0 * VBY * rn) < 120e6;
                     sa.vstride_in = sa.vstride_out = vsg;
@@ -998,7 +996,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
                             sa.out = (it & 1) ? x : y;
                             sa.alpha = alpha_g + gi;
                             sa.alphaf = alphaf_g + gi;
-                            e = op == 1                         ? launch_hop(sa)
+                            e = op == 1 && !whole               ? launch_hop(sa)
                                 : col                           ? launch_step_col(sa)
                                 : kern == TLS_KERNEL_MRHS_ROWS  ? launch_step_rows(sa, ctx->d_err)
                                 : kern == TLS_KERNEL_MRHS_ZM    ? launch_step_zm(sa)
@@ -1015,7 +1013,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
             if (e == cudaSuccess) {
                 if (il)
                     e = launch_unpack_il(result, storage, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn,
-                                         col ? cp.nvg : rn, 0, st, col);
+                                         col ? cp.nvg : rn, 0, st, col, whole);
                 else
                     e = launch_unpack_vectors(result, storage, vsg, dst_g, io_prec, vsites, g, gg->L, t_rel0, ns, gn, st);
                 ++launches;

@@ -121,9 +121,9 @@ inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby
 }
 
 // The same for the row kernel (k_ilt.cuh): 0.03 + 0.0105 n ns per site for n vectors
-// in fours (0.0125 n above 24), 0.02 + 0.015 n otherwise (48^3 x 32: 3 / 5 / 12 / 24 /
-// 72 vectors 224 / 394 / 578 / 1018 / 3510 us; 64^3 x 24: 8 / 24 vectors 595 / 1624
-// us), 1.75 times that where its TMA copies do not apply (50^3 x 16, 24 vectors: 884
+// in fours (0.0125 n above 24, 0.0145 n where a row's vectors take several CTAs), 0.02 +
+// 0.015 n otherwise (48^3 x 32: 3 / 5 / 12 / 24 / 72 vectors 224 / 394 / 578 / 1018 / 3510
+// us; 64^3 x 24: 8 / 24 vectors 595 / 1624 us; rows of 48, 24 vectors 0.0170 n), 1.75 times that where its TMA copies do not apply (50^3 x 16, 24 vectors: 884
 // us), with the arithmetic of the W formats shared by four vectors (24 vectors at
 // 48^3 x 32, row / column kernel: f32-18 1018 / 927, f32-12 1103 / 1065, f32-8 1699 /
 // above 2600, 16-bit vectors with f32-18 1203 / 1037, with f16-12 1393 / 1414 us).
@@ -135,7 +135,8 @@ inline double row_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb
 {
     const int n = (nvec + 1) & ~1;
     const double fmt = wb == 48 ? 1.08 : wb == 32 ? 1.65 : wb == 24 ? 1.15 : 1.0;
-    const double site = n % 4 ? 0.02 + 0.015 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
+    const bool split = n / 4 * g.hx > 256;  // the vectors of a row take several CTAs
+    const double site = n % 4 ? 0.02 + 0.015 * n : split ? 0.0145 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
     const bool tma = (g.hx * (wb % 16)) % 16 == 0;
     const double us = (double)nblk * g.Vs * site * 1e-3 * (tma ? 1.0 : 1.75) * (vby == 16 ? 1.2 : 1.0) * fmt;
     return std::max(us, row_ctas(g, nblk) * 1e-3) + 2;

@@ -25,6 +25,8 @@
 // halo) and the W rows of plane z0 + u; plane k uses unit k (W of the plane,
 // psi(k+1)) and unit k - 1 (psi of the plane's x and y neighbours, W_z(k-1)).
 //
+// HOP: the one-link step on whole slices (slice_geom), in which its hops are +-1 steps too.
+//
 // Every wait is bounded: one that runs out sets DERR_TIMEOUT and the CTA's
 // abort flag; the producer then waits (bounded) for its copies in flight
 // before the CTA ends.
@@ -122,7 +124,7 @@ __device__ __forceinline__ ColTile col_tile(int tile, int ngrp, const ColPlan &p
     return t;
 }
 
-template <int VP, int WF, bool ACT>
+template <int VP, int WF, bool ACT, bool HOP = false>
 __global__ void __launch_bounds__(kColMaxThreads, 1)
     k_step_col(const char *__restrict__ W, const char *__restrict__ in, char *__restrict__ out,
                const float *__restrict__ alphaf, const int *__restrict__ active, SubGeom g, ColPlan p, int64_t gstride,
@@ -389,8 +391,8 @@ __global__ void __launch_bounds__(kColMaxThreads, 1)
                 const float2 m6 = make_float2(-6.f, -6.f);
 #pragma unroll
                 for (int r = 0; r < 3; ++r) {
-                    re[r] = __ffma2_rn(a2, __ffma2_rn(m6, cR[r], aR[r]), cR[r]);
-                    im[r] = __ffma2_rn(a2, __ffma2_rn(m6, cI[r], aI[r]), cI[r]);
+                    re[r] = __ffma2_rn(a2, HOP ? aR[r] : __ffma2_rn(m6, cR[r], aR[r]), cR[r]);
+                    im[r] = __ffma2_rn(a2, HOP ? aI[r] : __ffma2_rn(m6, cI[r], aI[r]), cI[r]);
                 }
                 if (on0 && on1) {
                     if constexpr (VP == P_F32) {
@@ -446,6 +448,9 @@ template <int VP, int WF> cudaError_t col_launch(const StepArgs &a)
         p.smem = 128 + p.units * (p.recB + p.wB);
         const int64_t gstride = (int64_t)a.nblk * a.g.Ps * p.nvg * vfmt_bytes(VP);
         auto kern = a.active ? k_step_col<VP, WF, true> : k_step_col<VP, WF, false>;
+        if constexpr (WF == W_F32_18) {
+            if (a.hop) kern = k_step_col<VP, WF, false, true>;
+        }
         // always the same value: the attribute belongs to the function, other threads may launch it too
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kColMaxSmem);
         int occ = 0;

@@ -36,6 +36,9 @@
 // planes ahead in launch order, so their first DRAM touch happens before the
 // CTA that needs them waits for it.
 //
+// HOP: the one-link step (no -6 psi) on whole slices (slice_geom), in which its hops are +-1
+// steps too.
+//
 // The wait is bounded: if it runs out the CTA sets DERR_TIMEOUT, waits once
 // more (bounded) for its own copies in flight and returns without writing.
 #pragma once
@@ -125,7 +128,7 @@ __device__ __forceinline__ void ilt_prefetch_ahead(const char *__restrict__ W, c
 // One thread's part of a row: site x' = k of row (blk, zq, yq), vector units
 // t of T (VB vectors each), W rows staged at ws.  pl holds the records of the
 // first hop (requested before the wait on the copies).
-template <int VP, int WF, int VB, bool ACT, bool PF = false> struct IltSite {
+template <int VP, int WF, int VB, bool ACT, bool PF = false, bool HOP = false> struct IltSite {
     int nb[6];  // the six hops in the order of site_step
     int i;
     const char *rin;
@@ -450,8 +453,8 @@ template <int VP, int WF, int VB, bool ACT, bool PF = false> struct IltSite {
             const float2 a2 = *reinterpret_cast<const float2 *>(alphaf + v0);
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
-                pre[j][r] = __ffma2_rn(a2, __ffma2_rn(m6, pre[j][r], accR[j][r]), pre[j][r]);
-                pim[j][r] = __ffma2_rn(a2, __ffma2_rn(m6, pim[j][r], accI[j][r]), pim[j][r]);
+                pre[j][r] = __ffma2_rn(a2, HOP ? accR[j][r] : __ffma2_rn(m6, pre[j][r], accR[j][r]), pre[j][r]);
+                pim[j][r] = __ffma2_rn(a2, HOP ? accI[j][r] : __ffma2_rn(m6, pim[j][r], accI[j][r]), pim[j][r]);
             }
         }
         char *so = rout + (unsigned)i * rstride;
@@ -570,13 +573,14 @@ __device__ __forceinline__ bool ilt_wait(uint64_t *bar, unsigned parity)
 // RB (one vector group per row, vector pairs): the row's own records are
 // copied into shared memory with the W rows, and the x neighbours and the
 // centre are read from there.
-template <int VP, int WF, int VB, bool ACT, int MAXT, int MINB, bool PF = false, bool RB = false>
+template <int VP, int WF, int VB, bool ACT, int MAXT, int MINB, bool PF = false, bool RB = false, bool HOP = false>
 __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict__ W, const char *__restrict__ in,
                                                         char *__restrict__ out, const float *__restrict__ alphaf,
                                                         const int *__restrict__ active, SubGeom g, int nvec, int *err,
                                                         int pfd)
 {
     static_assert(!RB || (VB % 2 == 0 && !PF), "row staging: vector pairs, no next-hop prefetch");
+    static_assert(!HOP || (VB % 2 == 0 && VB <= 4), "one-link step: vector pairs");
     static_assert(VP != P_F64, "packed FP32 pairs only");
     extern __shared__ __align__(128) unsigned char ilt_sm[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(ilt_sm);
@@ -630,7 +634,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict_
     const int k = threadIdx.y;                           // x' of this thread's site
     const int t = blockIdx.x * blockDim.x + threadIdx.x;  // vector unit over the whole site
     const int T = nvec / VB;
-    IltSite<VP, WF, VB, ACT, PF> st;
+    IltSite<VP, WF, VB, ACT, PF, HOP> st;
     if constexpr (RB) {
         st.rbuf = rbuf;
         st.rcs = g.hx * nvec;
@@ -696,6 +700,13 @@ template <int VP, int WF, int VB> cudaError_t ilt_launch(const StepArgs &a)
             return launch_dep(a.dep, act ? kern_act : kern, grid, block, sm, a.stream, a.W, a.in, a.out, a.alphaf, a.active,
                               a.g, a.nvec, a.err, pfd);
         };
+        if (a.hop) {
+            if constexpr (WF == W_F32_18 && (VB == 2 || VB == 4)) {
+                constexpr auto kern = k_step_ilt<VP, WF, VB, false, 256, 3, false, false, true>;
+                return go(kern, kern, smem);
+            }
+            return cudaErrorNotSupported;
+        }
         if constexpr (VB % 2 == 0) {
             // tile[1] = 8: the row's own records staged with the W rows (one vector group per row)
             const int smem_rb = smem + a.g.hx * a.nvec * vfmt_bytes(VP);

@@ -300,6 +300,29 @@ __global__ void __launch_bounds__(128, 4) k_build_split(const double2 *__restric
     }
 }
 
+// The links rounded to FP32, a slice as one block of gc with its sites in canonical order.
+__global__ void __launch_bounds__(128) k_links_slices(const double2 *__restrict__ Up, char *__restrict__ L1, SubGeom g,
+                                                      SubGeom gc, int64_t total)
+{
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= total) return;
+    const int c = (int)(idx % gc.Vs);
+    const int64_t r = idx / gc.Vs;
+    const int d = (int)(r % 3), t = (int)(r / 3);
+    const int x = c % gc.hx, y = c / gc.hx % gc.hy, z = c / gc.hx / gc.hy;
+    const int sub = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
+    const int i = ((z >> 1) * g.hy + (y >> 1)) * g.hx + (x >> 1);
+    const double2 *A = Up + ((int64_t)(t * 8 + sub) * 3 + d) * 9 * g.Ps + i;
+    double w[18];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const double2 v = A[k * g.Ps];
+        w[2 * k] = v.x;
+        w[2 * k + 1] = v.y;
+    }
+    WFmt<W_F32_18>::store(L1 + ((int64_t)t * 3 + d) * gc.Ps * wfmt_bytes(W_F32_18), gc.Ps, c, w);
+}
+
 template <int WF>
 __global__ void k_export_twolink(const char *__restrict__ W, double *__restrict__ out, SubGeom g, int Lx, int Ly,
                                  int Lz, int64_t total)
@@ -662,7 +685,7 @@ struct PairArgs {
     int Lx, Ly, Lz, t_first;
     int nvec, rec_n, rec_v0;
     int64_t gstride;       // bytes between the fields of two groups
-    bool rc;
+    bool rc, whole;        // rows contiguous; blocks are whole slices
 };
 
 template <typename IO, int VP, bool PACK, bool AL>
@@ -675,7 +698,7 @@ __global__ void __launch_bounds__(256) k_move_pairs(std::conditional_t<PACK, con
     const int nv = min(a.nvec - first, a.rec_n);
     const int u0 = a.rec_v0 >> 1, T = ((a.rec_v0 + nv + 1) >> 1) - u0;
     const int sub0 = ((y & 1) << 1) | ((z & 1) << 2);
-    const int r = ((z >> 1) * g.hy + (y >> 1)) * g.hx;
+    const int r = a.whole ? (z * g.hy + y) * g.hx : ((z >> 1) * g.hy + (y >> 1)) * g.hx;
     const int64_t site0 = (((int64_t)(a.t_first + ts) * a.Lz + z) * a.Ly + y) * a.Lx;
     const int64_t sb = (int64_t)a.rec_n * VRec<VP>::SB;
     const int cs = (int)((a.rc ? g.hx : g.Ps) * a.rec_n);
@@ -684,8 +707,9 @@ __global__ void __launch_bounds__(256) k_move_pairs(std::conditional_t<PACK, con
         const int x = k / T, u = u0 + k - x * T;
         const int v0 = 2 * u - a.rec_v0;
         const bool on0 = v0 >= 0, on1 = v0 + 1 < nv;
-        auto *s = recs + blockIdx.z * a.gstride + ((int64_t)(ts * 8 + (sub0 | (x & 1))) * g.Ps * a.rec_n) * vfmt_bytes(VP) +
-                  (row + (x >> 1)) * sb;
+        const int b = a.whole ? ts : ts * 8 + (sub0 | (x & 1));
+        auto *s = recs + blockIdx.z * a.gstride + ((int64_t)b * g.Ps * a.rec_n) * vfmt_bytes(VP) +
+                  (row + (a.whole ? x : x >> 1)) * sb;
         auto *p = canon + ((int64_t)(first + v0) * a.vs + site0 + x) * 6;
         const int64_t next = a.vs * 6;
         cpx<float> q[2][3];
@@ -812,9 +836,17 @@ cudaError_t launch_build_links(const double *Up, char *L1, int wfmt, const SubGe
     const unsigned nb = nblocks(total, 128);
     switch (wfmt) {
     case W_F64_18: k_build_twolink<W_F64_18, true><<<nb, 128, 0, s>>>(u, L1, g, total, nullptr); break;
-    case W_F32_18: k_build_twolink<W_F32_18, true><<<nb, 128, 0, s>>>(u, L1, g, total, nullptr); break;
     default: return cudaErrorNotSupported;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_build_links_slices(const double *Up, char *L1, const SubGeom &g, const SubGeom &gc, int nsl,
+                                      cudaStream_t s)
+{
+    const int64_t total = (int64_t)nsl * 3 * gc.Vs;
+    if (total == 0) return cudaSuccess;
+    k_links_slices<<<nblocks(total, 128), 128, 0, s>>>(reinterpret_cast<const double2 *>(Up), L1, g, gc, total);
     return cudaGetLastError();
 }
 
@@ -901,36 +933,37 @@ static cudaError_t move_f64(bool pack, const void *canon, int64_t vs, char *recs
 
 template <bool PACK>
 static cudaError_t move_il(const void *canon, int io_prec, int64_t vs, char *recs, int prec, const SubGeom &g,
-                           const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0, cudaStream_t s, bool rc)
+                           const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0, cudaStream_t s, bool rc, bool whole)
 {
     if ((int64_t)nsl * 8 * g.Vs == 0 || nvec == 0) return cudaSuccess;
     const int ngrp = rc && rec_v0 == 0 ? (nvec + rec_n - 1) / rec_n : 1;
     if (nvec > 256 || rec_v0 < 0 || (ngrp == 1 && rec_v0 + nvec > rec_n)) return cudaErrorInvalidValue;
     if (io_prec != P_F64 && io_prec != P_F32) return cudaErrorNotSupported;
     if (prec == P_F64) {
-        if (rc) return cudaErrorNotSupported;
+        if (rc || whole) return cudaErrorNotSupported;
         return io_prec == P_F64
                    ? move_f64<double>(PACK, canon, vs, recs, g, L, t_first, nsl, nvec, rec_n, rec_v0, s)
                    : move_f64<float>(PACK, canon, vs, recs, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
     }
-    const PairArgs a{vs, L[0], L[1], L[2], t_first, nvec, rec_n, rec_v0, (int64_t)nsl * 8 * g.Ps * rec_n * vfmt_bytes(prec), rc};
+    const PairArgs a{vs, L[0], L[1], L[2], t_first, nvec, rec_n, rec_v0, (int64_t)nsl * (whole ? 1 : 8) * g.Ps * rec_n * vfmt_bytes(prec),
+                     rc, whole};
     return io_prec == P_F64 ? move_pairs<double, PACK>(canon, recs, prec, g, nsl, ngrp, a, s)
                             : move_pairs<float, PACK>(canon, recs, prec, g, nsl, ngrp, a, s);
 }
 
 cudaError_t launch_pack_il(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                            const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                           cudaStream_t s, bool rc)
+                           cudaStream_t s, bool rc, bool whole)
 {
-    return move_il<true>(src, io_prec, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s, rc);
+    return move_il<true>(src, io_prec, src_vstride_sites, dst, prec, g, L, t_first, nsl, nvec, rec_n, rec_v0, s, rc, whole);
 }
 
 cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, int64_t dst_vstride_sites,
                              const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                             cudaStream_t s, bool rc)
+                             cudaStream_t s, bool rc, bool whole)
 {
     return move_il<false>(dst, io_prec, dst_vstride_sites, const_cast<char *>(src), prec, g, L, t_first, nsl, nvec, rec_n,
-                          rec_v0, s, rc);
+                          rec_v0, s, rc, whole);
 }
 
 cudaError_t launch_norm_partials(const void *base, int io_prec, int64_t vstride_sites, int64_t slice_sites, int nsl,

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(32) k_step_row3(const char *__restrict__ W, co
 // per vector is the same sequence as site_step, so results are bitwise equal
 // to the planar kernels.
 // --------------------------------------------------------------------------
-template <int VP, int WF, int VB>
+template <int VP, int WF, int VB, bool HOP = false>
 __device__ __forceinline__ void step_il_body(const char *__restrict__ W, const char *__restrict__ in,
                                              char *__restrict__ out, const double *__restrict__ alpha,
                                              const int *__restrict__ active, const SubGeom &g, int nvec)
@@ -264,8 +264,8 @@ __device__ __forceinline__ void step_il_body(const char *__restrict__ W, const c
         const R a = (R)alpha[il_vec<VP, VB>(t, T, k)];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            o[k][q].re = fma(a, fma(R(-6), c[k][q].re, acc[k][q].re), c[k][q].re);
-            o[k][q].im = fma(a, fma(R(-6), c[k][q].im, acc[k][q].im), c[k][q].im);
+            o[k][q].re = fma(a, HOP ? acc[k][q].re : fma(R(-6), c[k][q].re, acc[k][q].re), c[k][q].re);
+            o[k][q].im = fma(a, HOP ? acc[k][q].im : fma(R(-6), c[k][q].im, acc[k][q].im), c[k][q].im);
         }
         if (!on[k]) {
 #pragma unroll
@@ -286,12 +286,12 @@ __device__ __forceinline__ void step_il_body(const char *__restrict__ W, const c
     }
 }
 
-template <int VP, int WF, int VB>
+template <int VP, int WF, int VB, bool HOP = false>
 __global__ void __launch_bounds__(256) k_step_il(const char *__restrict__ W, const char *__restrict__ in,
                                                  char *__restrict__ out, const double *__restrict__ alpha,
                                                  const int *__restrict__ active, SubGeom g, int nvec)
 {
-    step_il_body<VP, WF, VB>(W, in, out, alpha, active, g, nvec);
+    step_il_body<VP, WF, VB, HOP>(W, in, out, alpha, active, g, nvec);
 }
 
 // The same kernel held to 64 registers (CTAs of at most 128 threads, 8 per
@@ -1073,6 +1073,16 @@ template <int VP, int WF, int VB, bool ONLYX = false> cudaError_t step_il_launch
     spb = std::max(1, std::min(spb, cap / tx));
     spb = std::min(spb, a.g.hx);  // a strip never spans more than one row
     // the packed kernel also serves slot batches (active table); the other staged forms do not
+    if (a.hop) {  // one-link step on rows the row kernel does not take
+        if constexpr (WF == W_F32_18 && !ONLYX) {
+            if (tx * spb > cap) return cudaErrorInvalidConfiguration;
+            const dim3 block(tx, spb), grid((a.g.hx + spb - 1) / spb, a.g.hy, (unsigned)a.g.hz * a.nblk);
+            if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
+            k_step_il<VP, WF, VB, true><<<grid, block, 0, a.stream>>>(a.W, a.in, a.out, a.alpha, nullptr, a.g, a.nvec);
+            return cudaGetLastError();
+        }
+        return cudaErrorNotSupported;
+    }
     const bool packed = (a.tile[1] == 2 || ilt || ((a.tile[1] == 3 || a.tile[1] == 5) && a.active == nullptr)) &&
                         a.alphaf && VP != P_F64;
     const bool staged = a.tile[1] > 0 && a.active == nullptr && a.alphaf;

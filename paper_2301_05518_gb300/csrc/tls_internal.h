@@ -31,6 +31,7 @@ struct StepArgs {
     int tile[3];           // interleaved kernel: sites per CTA along x', y', z' (0 = a strip along x')
     int *err;              // device error word (kernels with bounded waits); nullable for the others
     int num_sms;           // of the device (persistent CTAs of the column kernel)
+    bool hop;              // one-link step: psi + alpha H psi (no -6 psi); W is the link field on whole slices
     bool dep;              // short steps: start while the step before drains (launch.cuh)
     cudaStream_t stream;
 };
@@ -84,7 +85,7 @@ cudaError_t launch_step_il(const StepArgs &a);
 cudaError_t launch_step_col(const StepArgs &a);
 // The same step marching along z' with a register window (interleaved layout, active unused).
 cudaError_t launch_step_zm(const StepArgs &a);
-// One-link Gaussian smearing step psi + alpha H psi (interleaved layout; W = the link field).
+// One-link Gaussian smearing step psi + alpha H psi in FP64 (interleaved layout; W = the link field).
 cudaError_t launch_hop(const StepArgs &a);
 // The same step with TMA row staging in shared memory (k_rows.cuh); err gets
 // DERR_TIMEOUT if a bounded wait runs out.  rows_applicable says whether the
@@ -108,10 +109,6 @@ cudaError_t launch_step_col_f32(const StepArgs &a);
 cudaError_t launch_step_col_f16(const StepArgs &a);
 cudaError_t launch_step_col_bf16(const StepArgs &a);
 cudaError_t launch_step_zm_f64(const StepArgs &a);
-cudaError_t launch_hop_f64(const StepArgs &a);
-cudaError_t launch_hop_f32(const StepArgs &a);
-cudaError_t launch_hop_f16(const StepArgs &a);
-cudaError_t launch_hop_bf16(const StepArgs &a);
 cudaError_t launch_step_zm_f32(const StepArgs &a);
 cudaError_t launch_step_zm_f16(const StepArgs &a);
 cudaError_t launch_step_zm_bf16(const StepArgs &a);
@@ -136,6 +133,9 @@ cudaError_t launch_build_twolink(const double *Up, char *W, int wfmt, const SubG
                                  cudaStream_t s);
 // The one-link field: U itself rounded into a W format (same planes as W).
 cudaError_t launch_build_links(const double *Up, char *L1, int wfmt, const SubGeom &g, int nblk, cudaStream_t s);
+// The same in FP32 on whole slices: one block per slice, sites in canonical order (gc = slice_geom).
+cudaError_t launch_build_links_slices(const double *Up, char *L1, const SubGeom &g, const SubGeom &gc, int nsl,
+                                      cudaStream_t s);
 // One APE step on the packed spatial links: out = P((1-a) U + (a/4) staples) (k_ape.cu).
 cudaError_t launch_ape_step(const double *U, double *out, const SubGeom &g, int nblk, double a, int *err,
                             cudaStream_t s);
@@ -145,12 +145,13 @@ cudaError_t launch_export_twolink(const char *W, int wfmt, double *out, const Su
 // (0 <= v < nvec) goes to / comes from record rec_v0 + v.  rc (FP32 and 16-bit): the colour
 // planes are those of each x'-row instead of the block's, so that a row is contiguous, and
 // with rec_v0 = 0 the vectors go to successive fields of rec_n each (column kernel).
+// whole (FP32 and 16-bit): g is slice_geom, a block is a slice in canonical order.
 cudaError_t launch_pack_il(const void *src, int io_prec, int64_t src_vstride_sites, char *dst, int prec,
                            const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                           cudaStream_t s, bool rc = false);
+                           cudaStream_t s, bool rc = false, bool whole = false);
 cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, int64_t dst_vstride_sites,
                              const SubGeom &g, const int L[4], int t_first, int nsl, int nvec, int rec_n, int rec_v0,
-                             cudaStream_t s, bool rc = false);
+                             cudaStream_t s, bool rc = false, bool whole = false);
 // FP64 |psi|^2 partial sums of nvec canonical vectors (vector v at base + v * vstride
 // sites), kNormPartsPerSlice per (vector, slice) over nsl slices of slice_sites sites:
 // partial (v, s, p) at partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].

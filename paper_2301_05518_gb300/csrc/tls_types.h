@@ -45,6 +45,15 @@ struct SubGeom {
     int64_t Ps;      // plane stride (Vs rounded up to 32)
 };
 
+// The one-link hops connect the sublattices, so their FP32 and 16-bit fields take a slice whole:
+// one block of Lx x Ly x Lz sites in canonical order, in which a hop is a +-1 step.
+TLS_HD inline SubGeom slice_geom(const int L[4])
+{
+    SubGeom g{L[0], L[1], L[2], L[0] * L[1] * L[2], 0};
+    g.Ps = ((int64_t)g.Vs + 31) / 32 * 32;
+    return g;
+}
+
 // Device error word bits.
 enum DevErr {
     DERR_BOUNDS = 1,      // an index check failed (checked builds)
