@@ -121,7 +121,7 @@ inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby
 }
 
 // The same for the row kernel (k_ilt.cuh): 0.03 + 0.0105 n ns per site for n vectors
-// in fours (0.0125 n above 24, 0.0145 n where a row's vectors take several CTAs), 0.02 +
+// in fours (0.0125 n above 24, 0.0165 n where a row's vectors take several CTAs), 0.02 +
 // 0.015 n otherwise (48^3 x 32: 3 / 5 / 12 / 24 / 72 vectors 224 / 394 / 578 / 1018 / 3510
 // us; 64^3 x 24: 8 / 24 vectors 595 / 1624 us; rows of 48, 24 vectors 0.0170 n), 1.75 times that where its TMA copies do not apply (50^3 x 16, 24 vectors: 884
 // us), with the arithmetic of the W formats shared by four vectors (24 vectors at
@@ -136,7 +136,7 @@ inline double row_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb
     const int n = (nvec + 1) & ~1;
     const double fmt = wb == 48 ? 1.08 : wb == 32 ? 1.65 : wb == 24 ? 1.15 : 1.0;
     const bool split = n / 4 * g.hx > 256;  // the vectors of a row take several CTAs
-    const double site = n % 4 ? 0.02 + 0.015 * n : split ? 0.0145 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
+    const double site = n % 4 ? 0.02 + 0.015 * n : split ? 0.0165 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
     const bool tma = (g.hx * (wb % 16)) % 16 == 0;
     const double us = (double)nblk * g.Vs * site * 1e-3 * (tma ? 1.0 : 1.75) * (vby == 16 ? 1.2 : 1.0) * fmt;
     return std::max(us, row_ctas(g, nblk) * 1e-3) + 2;
