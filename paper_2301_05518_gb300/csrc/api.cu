@@ -738,7 +738,10 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     if (col_ok && planned) {
         double us = 0;
         const double row_us = row_estimate(g, nblk, col_n, VBY, wfmt_bytes(fmt));
-        const bool have_col = col_plans(g, nblk, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1) > 0;
+        // under an HBM cap only groups without padding: buffers stay as large as the row kernel's
+        const bool exact = ctx->cap != 0;
+        const bool have_col =
+            col_plans(g, nblk, exact ? (col_n + 1) & ~1 : col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1, exact) > 0;
         if (op == 0 && planar_ok(g, nblk, nvec, wfmt_bytes(fmt)) &&
             planar_estimate(g, nblk, nvec, VBY, wfmt_bytes(fmt)) < (have_col ? std::min(us, row_us) : row_us)) {
             tile[1] = 10;
@@ -798,23 +801,10 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     auto packed_of = [&](int n) {  // records per site in the packed buffers
         return col ? (n + cp.nvg - 1) / cp.nvg * cp.nvg : il_layout ? rec_of(n) : n;
     };
-    s = ensure(ctx, ctx->A, (size_t)vs * packed_of(G), "tls_smear: vector buffer A");
-    if (s == TLS_OK) s = ensure(ctx, ctx->B, (size_t)vs * packed_of(G), "tls_smear: vector buffer B");
-    if (s != TLS_OK && col && packed_of(G) > rec_of(G)) {  // without the padding of the vector groups
-        col = false;
-        vb = row_tile(g, nblk, col_n, VBY, tile);
-        if (G0 % vb != 0) vb = default_il_vb(storage, G0);
-        s = ensure(ctx, ctx->A, (size_t)vs * packed_of(G), "tls_smear: vector buffer A");
-        if (s == TLS_OK) s = ensure(ctx, ctx->B, (size_t)vs * packed_of(G), "tls_smear: vector buffer B");
-    }
     // alpha per vector in FP64, then the same rounded to FP32 (read by the FP32-arithmetic
-    // kernels); one more entry of each for a padding record
-    const int nalpha = nvec + std::max(1, col ? cp.nvg : 0);
-    const size_t alpha_bytes = sizeof(double) * nalpha + sizeof(float) * nalpha;
-    if (s == TLS_OK) s = ensure(ctx, ctx->alpha, alpha_bytes, "tls_smear: alpha");
-    if (s == TLS_OK && norms_out)
-        s = ensure(ctx, ctx->partials, sizeof(double) * kNormPartsPerSlice * nsl * nvec, "tls_smear: partials");
-    if (s == TLS_OK && norms_out) s = ensure(ctx, ctx->norms, sizeof(double) * nvec, "tls_smear: norms");
+    // kernels); entries for the padding records of the last group too
+    int nalpha = 0;
+    size_t alpha_bytes = 0;
     // Host vectors go through slice groups of about kGroupBytes in up to three
     // rotating staging slots, so that copies in and out overlap the smearing
     // of other groups.  The persistent kernel takes all slices in one group.
@@ -829,7 +819,28 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         }
         nslot = std::min(ngroup, 3);
         slot_bytes = (io_slice_bytes * tg * nvec + 255) / 256 * 256;
-        if (s == TLS_OK) s = ensure(ctx, ctx->staging, slot_bytes * nslot, "tls_smear: host staging");
+    }
+    auto workspace = [&]() -> tls_status {
+        const int last = (nvec - 1) / G * G;  // first vector of the last group
+        nalpha = std::max(nvec + 1, last + packed_of(nvec - last));
+        alpha_bytes = (sizeof(double) + sizeof(float)) * nalpha;
+        tls_status r = ensure(ctx, ctx->A, (size_t)vs * packed_of(G), "tls_smear: vector buffer A");
+        if (r == TLS_OK) r = ensure(ctx, ctx->B, (size_t)vs * packed_of(G), "tls_smear: vector buffer B");
+        if (r == TLS_OK) r = ensure(ctx, ctx->alpha, alpha_bytes, "tls_smear: alpha");
+        if (r == TLS_OK && norms_out)
+            r = ensure(ctx, ctx->partials, sizeof(double) * kNormPartsPerSlice * nsl * nvec, "tls_smear: partials");
+        if (r == TLS_OK && norms_out) r = ensure(ctx, ctx->norms, sizeof(double) * nvec, "tls_smear: norms");
+        if (r == TLS_OK && staged) r = ensure(ctx, ctx->staging, slot_bytes * nslot, "tls_smear: host staging");
+        return r;
+    };
+    s = workspace();
+    if (s != TLS_OK && col && packed_of(G) > rec_of(G)) {  // once more without the padding of the vector groups
+        col = false;
+        vb = row_tile(g, nblk, col_n, VBY, tile);
+        if (G0 % vb != 0) vb = default_il_vb(storage, G0);
+        release(ctx, ctx->A);
+        release(ctx, ctx->B);
+        s = workspace();
     }
     if (s != TLS_OK) return s;
     if (ctx->h_alpha_n < (size_t)nalpha) {

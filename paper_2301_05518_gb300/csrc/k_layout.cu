@@ -10,6 +10,8 @@
 //
 // Packed U layout: block b = t * 8 + sub, direction d, entry k = 0..8:
 //   Up[((b * 3 + d) * 9 + k) * Ps + i]  (double2 = one complex entry)
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -490,24 +492,27 @@ __global__ void k_unpack_il(const char *__restrict__ src, IO *__restrict__ dst, 
     }
 }
 
-// Partial sums of |psi|^2 of canonical vectors, per (vector, slice, part):
-// CTA (s * kNormPartsPerSlice + p, v) takes a fixed strided subset of the
-// reals of slice s of vector v, so each partial depends only on its own slice
-// and the sum order is fixed.  Partial (v, s, p) goes to
-// partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].
+// Partial sums of |psi|^2 of canonical vectors, per (vector, slice, part): a cluster of
+// kNormSplit CTAs takes a fixed strided subset of the reals of slice s of vector v, so each
+// partial depends only on its own slice and the sum order is fixed.  Partial (v, s, p) goes to
+// partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].  Bound by the FP64 adds of
+// the SMs in use: with norms of one slice of 48^3, 3 vectors, a call takes 22 us longer, 38 with one
+// CTA per partial (and as long with 64 partials per slice, which take four times the scratch).
+constexpr int kNormSplit = 4;
 template <typename IO>
-__global__ void __launch_bounds__(256) k_norm_partials(const IO *__restrict__ base, int64_t vstride, int64_t slice_sites,
-                                                       double *__restrict__ partials, int64_t part_stride,
-                                                       int64_t part_off)
+__global__ void __cluster_dims__(kNormSplit, 1, 1) __launch_bounds__(256)
+    k_norm_partials(const IO *__restrict__ base, int64_t vstride, int64_t slice_sites, double *__restrict__ partials,
+                    int64_t part_stride, int64_t part_off)
 {
+    constexpr int kCtas = kNormPartsPerSlice * kNormSplit;  // of a slice
     __shared__ double red[256];
     const int v = blockIdx.y;
-    const int sl = blockIdx.x / kNormPartsPerSlice, part = blockIdx.x - sl * kNormPartsPerSlice;
+    const int sl = blockIdx.x / kCtas, part = blockIdx.x - sl * kCtas;
     const IO *p = base + ((int64_t)v * vstride + (int64_t)sl * slice_sites) * 6;
     const int64_t n = slice_sites * 6;
     double acc = 0.0;
 #pragma unroll 8
-    for (int64_t k = (int64_t)part * blockDim.x + threadIdx.x; k < n; k += (int64_t)kNormPartsPerSlice * blockDim.x) {
+    for (int64_t k = (int64_t)part * blockDim.x + threadIdx.x; k < n; k += (int64_t)kCtas * blockDim.x) {
         const double x = (double)p[k];
         acc = fma(x, x, acc);
     }
@@ -517,7 +522,14 @@ __global__ void __launch_bounds__(256) k_norm_partials(const IO *__restrict__ ba
         if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partials[(int64_t)v * part_stride + part_off + blockIdx.x] = red[0];
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();
+    if (cl.block_rank() == 0 && threadIdx.x == 0) {
+        double sum = red[0];
+        for (int r = 1; r < kNormSplit; ++r) sum += *cl.map_shared_rank(red, r);
+        partials[(int64_t)v * part_stride + part_off + blockIdx.x / kNormSplit] = sum;
+    }
+    cl.sync();  // no CTA leaves while its sum is read
 }
 
 // Copies the interleaved records of one x'-row (hx sites starting at site r of
@@ -970,8 +982,8 @@ cudaError_t launch_norm_partials(const void *base, int io_prec, int64_t vstride_
                                  int nvec, double *partials, int64_t part_stride, int64_t part_off, cudaStream_t s)
 {
     if (nvec == 0 || nsl == 0) return cudaSuccess;
-    if ((int64_t)nsl * kNormPartsPerSlice > 0x7fffffff || nvec > 65535) return cudaErrorInvalidValue;
-    dim3 grid(nsl * kNormPartsPerSlice, nvec);
+    if ((int64_t)nsl * kNormPartsPerSlice * kNormSplit > 0x7fffffff || nvec > 65535) return cudaErrorInvalidValue;
+    dim3 grid(nsl * kNormPartsPerSlice * kNormSplit, nvec);
     if (io_prec == P_F64)
         k_norm_partials<double><<<grid, 256, 0, s>>>((const double *)base, vstride_sites, slice_sites, partials,
                                                       part_stride, part_off);

@@ -157,7 +157,7 @@ cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, 
 // partial (v, s, p) at partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].
 // A partial depends only on its slice, so slices may be summed in separate launches;
 // launch_reduce_norms(partials, part_stride, ...) then adds each vector's partials in order.
-const int kNormPartsPerSlice = 64;  // one slice of 48^3, 3 vectors: 36 us with 16, 20 us with 64 (the FP64 adds of a slice spread over more SMs)
+const int kNormPartsPerSlice = 16;
 cudaError_t launch_norm_partials(const void *base, int io_prec, int64_t vstride_sites, int64_t slice_sites, int nsl,
                                  int nvec, double *partials, int64_t part_stride, int64_t part_off, cudaStream_t s);
 // Canonical caller vectors (io_prec F64/F32, slices [t_first, t_first + nsl)) -> packed storage.

@@ -91,22 +91,23 @@ def test_planner_choice_bitwise_equals_single(ctx, T, dims, nvec, storage):
     ctx.free_gauge(gid)
 
 
-def test_padded_groups_do_not_cost_admission(T):
-    """A smear whose exact buffers fit under the HBM cap runs although the padded vector groups of
-    the column kernel would not fit."""
+@pytest.mark.parametrize("records,slack", [(50, 1 << 17), (60, 1 << 13)])
+def test_padded_groups_do_not_cost_admission(T, records, slack):
+    """A smear whose buffers fit under the HBM cap runs although the padded vector groups of the
+    column kernel (60 records), or what is allocated after them, would not fit."""
     dims, nvec = (16, 16, 16, 8), 49
-    exact = 2 * 50 * 24 * 16 ** 3 * 8          # two packed buffers of 50 records
+    bufs = 2 * records * 24 * 16 ** 3 * 8      # two packed buffers
     fixed = 3 * 144 * 16 ** 3 * 8 + 216 * 16 ** 3 * 8
-    with T.Context(0, hbm_cap_bytes=exact + fixed + (1 << 16)) as c:
+    with T.Context(0, hbm_cap_bytes=bufs + fixed + slack) as c:
         gid = c.load_gauge(synth.gauge_haar(dims, 55, nd=3).cuda(), 3, dims)
         c.build_twolink(gid, T.TLS_F32, 18)
-        c.tune_set(gid, nvec, T.TLS_F32, T.TLS_ALL_T, T.TLS_KERNEL_MRHS, 2, 0, (10, 9, 4 | 1 << 8))
+        c.tune_set(gid, nvec, T.TLS_F32, T.TLS_ALL_T, T.TLS_KERNEL_MRHS, 2, 0, (12, 9, 4 | 1 << 8))
         x = synth.gaussian_vectors(dims, nvec, 56, dtype=torch.complex64).cuda()
         want = x.clone()
         c.smear(gid, want[:7].contiguous(), T.TLS_F32, 7, 3, 0.6, kernel=T.TLS_KERNEL_SINGLE)
         one = want[7:8].contiguous()
         c.smear(gid, one, T.TLS_F32, 1, 3, 0.6, kernel=T.TLS_KERNEL_SINGLE)
-        c.smear(gid, x, T.TLS_F32, nvec, 3, 0.6)
+        c.smear(gid, x, T.TLS_F32, nvec, 3, 0.6, norms=True)
         assert torch.equal(x[7:8], one)
 
 
