@@ -78,6 +78,7 @@ PROFILED_TRAFFIC_PER_SITE = {
     ("mrhs", 4, (0, 2, 0)): 1337.3,  # k_step_ilx, profiles/k_step_ilx_64x64x64x4_24vec_f32.md
     ("mrhs", 4, (0, 6, 0)): 1337.3,  # k_step_ilt, profiles/k_step_ilt_64x64x64x4_24vec_f32.md
     ("mrhs", 4, (0, 6, -1)): 1337.7,  # k_step_ilt with the L2 prefetch, same profile
+    ("mrhs", 2, (12, 9, 262402)): 1382.6,  # k_step_col, profiles/k_step_col_64x64x64x4_24vec_f32.md
 }
 
 
@@ -781,7 +782,8 @@ def our_arm(args):
         result["build"] = {"ms": prof_last["ms_build"], "flops": build_flops,
                            "tflops": build_flops / (prof_last["ms_build"] / 1e3) / 1e12,
                            "frac_of_fp64_peak": build_flops / (prof_last["ms_build"] / 1e3) / 1e12 / peaks["fp64_tflops"],
-                           "peak_source": "measured (tls_peak_flops, FP64 FMA chains)"}
+                           "peak_source": "measured (tls_peak_flops, FP64 FMA chains)",
+                           "note": "products in FP32 slices, bit for bit the FP64 ones: may exceed the FP64 rate"}
         # APE smearing of the links (FP64, staples + projection onto SU(3)), one step
         gid = ctx.load_gauge(U, 4, dims, stream=stream)
         ctx.ape_smear(gid, 0.5, 1, stream=stream)

@@ -128,8 +128,7 @@ tls_status tls_build_twolink(tls_ctx *ctx, tls_gauge_id id, int wprec, int recon
 
 /* ---- one-link field (Sec. 2, Eq. 2: the links U_mu of the hopping term) -----
  * Stores the spatial links U_mu(x) themselves, rounded to nearest in `prec`
- * (TLS_F64 or TLS_F32), in the two-link field's layout, for
- * tls_smear_onelink.  keep_U = 0 releases the FP64 device copy of U.
+ * (TLS_F64 or TLS_F32), for tls_smear_onelink.  keep_U = 0 releases the FP64 device copy of U.
  * Errors: TLS_ERR_NOT_FOUND, TLS_ERR_STATE (U released), TLS_ERR_UNSUPPORTED. */
 tls_status tls_build_links(tls_ctx *ctx, tls_gauge_id id, int prec, int keep_U, void *stream);
 
