@@ -680,6 +680,10 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     const bool whole = op == 1 && storage != TLS_F64;
     const SubGeom g = whole ? slice_geom(gg->L) : gg->g;
     const int bps = whole ? 1 : 8;  // blocks per slice
+    // Vectors packed at a time.  The row and interleaved kernels take 32-bit byte offsets inside a
+    // block (colour plane or 16-bit records); a whole slice has eight times the sites of a block.
+    const int64_t off_b = (int64_t)g.Ps * (storage == TLS_F32 ? 8 : 16);
+    const int gmax = whole ? (int)std::max<int64_t>(2, std::min<int64_t>(256, (int64_t(1) << 32) / off_b) & ~1) : 256;
     const int nsl = timeslice < 0 ? gg->L[3] : 1;
     const int t_first = timeslice < 0 ? 0 : timeslice;
     const int nblk = nsl * bps;
@@ -727,7 +731,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     // The column kernel (tile[1] = 9) works on vector groups of tile[0], one interleaved field
     // behind the other; a shape it does not take goes to the planner.
     const bool col_ok = kern == TLS_KERNEL_MRHS && storage != TLS_F64;
-    const int col_n = std::min(nvec, 256);
+    const int col_n = std::min(nvec, gmax);
     ColPlan cp{};
     bool col = false;
     if (col_ok && tile[1] == 9) {
@@ -759,7 +763,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     // (computed, never unpacked).
     const bool pad_pairs = storage != TLS_F64;
     auto rec_of = [&](int n) { return pad_pairs ? (n + 1) & ~1 : n; };
-    const int G0 = rec_of(std::min(nvec, 256));
+    const int G0 = rec_of(std::min(nvec, gmax));
     if (kern == TLS_KERNEL_SINGLE) {
         vb = 1;
         if (threads <= 0) threads = 128;
@@ -788,7 +792,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         threads = 128;
     }
     const bool il_layout = !planar && (kern == TLS_KERNEL_MRHS || kern == TLS_KERNEL_MRHS_ROWS || kern == TLS_KERNEL_MRHS_ZM);
-    const int G = il_layout ? std::min(nvec, 256) : nvec;
+    const int G = il_layout ? std::min(nvec, gmax) : nvec;
 
     // Host vectors go through bulk copies (DMA) into a staging buffer.  On a
     // GB300 these measured faster than letting the layout kernels read and

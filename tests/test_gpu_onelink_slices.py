@@ -37,3 +37,21 @@ def test_onelink_on_slices_matches_oracle(dims, nvec, storage, t0):
     assert max(per_vector_rel_l2(got, want)) <= (2e-6 * N if storage == "F32" else 5e-3)
     sl = slice(None) if t0 < 0 else slice(t0, t0 + 1)
     assert np.allclose(norms, (np.abs(got[:, sl]) ** 2).reshape(nvec, -1).sum(1), rtol=1e-12, atol=0)
+
+
+def test_onelink_batch_past_32_bit_offsets():
+    """Rows too long for a CTA of the column or row kernel, and a batch whose records of one slice
+    pass 4 GiB: every vector as in a batch of two."""
+    from paper_2301_05518_gb300 import tls as T
+    dims, nvec = (520, 64, 64, 1), 132
+    with T.Context(0) as ctx:
+        gid = ctx.load_gauge(synth.gauge_haar(dims, 63, nd=3), 3, dims)
+        ctx.build_links(gid, T.TLS_F32)
+        torch.manual_seed(64)
+        x = torch.randn((nvec, 1, 64, 64, 520, 3), dtype=torch.complex64, device="cuda")
+        pairs = [x[v:v + 2].clone() for v in (0, 124, 126, 130)]
+        ctx.smear_onelink(gid, x, T.TLS_F32, nvec, 2, 0.05, storage=T.TLS_F16)
+        for v, y in zip((0, 124, 126, 130), pairs):
+            ctx.smear_onelink(gid, y, T.TLS_F32, 2, 2, 0.05, storage=T.TLS_F16)
+            assert torch.equal(x[v:v + 2], y), v
+        ctx.free_gauge(gid)
