@@ -120,7 +120,8 @@ tls_status tls_load_gauge(tls_ctx *ctx, const double *U, int nd, const int dims[
  * stored with `recon` reals per matrix (TLS_R18; TLS_R12 or TLS_R8 for FP32;
  * TLS_R12 for 16-bit).  W stays resident until tls_free_gauge.  keep_U = 0
  * releases the device copy of U after the build.  Rebuilding replaces W.
- * Errors: TLS_ERR_NOT_FOUND, TLS_ERR_STATE (U already released),
+ * Errors: TLS_ERR_NOT_FOUND, TLS_ERR_STATE (U already released, or serving
+ * jobs on the gauge have not finished: they read W),
  * TLS_ERR_UNSUPPORTED (combination), TLS_ERR_DEVICE (TLS_R8 met a matrix with
  * |W00| too close to 1 to parameterise), memory errors.                     */
 tls_status tls_build_twolink(tls_ctx *ctx, tls_gauge_id id, int wprec, int recon,

@@ -425,6 +425,9 @@ tls_status tls_build_twolink(tls_ctx *ctx, tls_gauge_id id, int wprec, int recon
     if (!gg->Up) return fail(TLS_ERR_STATE, "tls_build_twolink: the links of gauge %lld were released", (long long)id);
     const int wf = wfmt_of(wprec, recon);
     if (wf < 0) return fail(TLS_ERR_UNSUPPORTED, "tls_build_twolink: precision %d with %d reals", wprec, recon);
+    // the batches' rounds read W and their graphs hold its address
+    if (serve_gauge_in_use(ctx, id))
+        return fail(TLS_ERR_STATE, "tls_build_twolink: serving jobs still use gauge %lld", (long long)id);
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const int nblk = gg->L[3] * 8;

@@ -156,7 +156,9 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
 
 // The serving subsystem (serve.cpp).
 void serve_shutdown(tls_ctx *ctx);
-// True if serving still holds jobs on gauge `id`; otherwise drops its idle batches.
+// True if a submitted job on gauge `id` has not finished.  The caller holds ctx->mu.
+bool serve_gauge_in_use(tls_ctx *ctx, int64_t id);
+// The same; if not, drops the gauge's idle batches.
 bool serve_gauge_busy(tls_ctx *ctx, int64_t id);
 
 }  // namespace tls

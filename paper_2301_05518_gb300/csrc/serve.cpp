@@ -272,8 +272,8 @@ int try_admit(tls_ctx *ctx, Server *sv, Job *j)
     BatchKey key{j->d.gauge, j->d.storage, j->d.timeslice};
     Batch *b = nullptr;
     auto bit = sv->batches.find(key);
-    if (bit != sv->batches.end() && bit->second->used_slots() == 0 &&
-        (bit->second->W != gg.W || bit->second->wfmt != gg.wfmt)) {  // W was rebuilt since
+    if (bit != sv->batches.end() && (bit->second->W != gg.W || bit->second->wfmt != gg.wfmt)) {  // W was rebuilt since
+        if (bit->second->used_slots() > 0) return 1;  // its graphs hold the old field: not for new jobs
         destroy_batch(ctx, bit->second.get());
         sv->batches.erase(bit);
         bit = sv->batches.end();
@@ -567,15 +567,26 @@ void serve_shutdown(tls_ctx *ctx)
     ctx->server = nullptr;
 }
 
+bool serve_gauge_in_use(tls_ctx *ctx, int64_t id)
+{
+    Server *sv = ctx->server;
+    if (!sv) return false;
+    // All jobs, not the pending ones: the scheduler takes those off the list before it has the
+    // context lock, so a job between the two is in neither the list nor a batch.
+    std::lock_guard<std::mutex> lk(sv->m);
+    for (auto &kv : sv->jobs)
+        if (!kv.second->done && kv.second->d.gauge == id) return true;
+    return false;
+}
+
 bool serve_gauge_busy(tls_ctx *ctx, int64_t id)
 {
     Server *sv = ctx->server;
     if (!sv) return false;
+    if (serve_gauge_in_use(ctx, id)) return true;
     // The caller holds ctx->mu, so the scheduler is not admitting or launching;
     // sv->m keeps its idle check (any_busy) off the map while it changes.
     std::lock_guard<std::mutex> lk(sv->m);
-    for (Job *j : sv->pending)
-        if (j->d.gauge == id) return true;
     for (auto it = sv->batches.begin(); it != sv->batches.end();) {
         Batch *b = it->second.get();
         if (b->key.gauge == id) {
