@@ -738,8 +738,7 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     ColPlan cp{};
     bool col = false;
     if (col_ok && tile[1] == 9) {
-        col = col_shape(g, nblk, col_n, VBY, wfmt_bytes(fmt), tile[0], tile[2] & 255, std::max(1, (tile[2] >> 8) & 255),
-                        cp);
+        col = col_of_tile(g, nblk, col_n, VBY, wfmt_bytes(fmt), tile, cp);
         planned = !col;
     }
     if (col_ok && planned) {

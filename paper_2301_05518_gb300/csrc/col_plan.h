@@ -63,11 +63,15 @@ struct ColPlan {
     ColW w;
 };
 
-// The tile shape: nvg vectors per group, ny rows, nseg segments.  False: no fit.
-inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int nvg, int ny, int nseg, ColPlan &out)
+// The tile shape: nvg vectors per group, ny rows, nseg segments, at most `units` ring units (0: as
+// many as fit).  False: no fit.  Fewer than three units are no ring: a consumer keeps the unit
+// before the one it waits for, and the producer runs one further.
+inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int nvg, int ny, int nseg, int units,
+                      ColPlan &out)
 {
     ColPlan p{};
     if (nvg < 2 || (nvg & 1) || ny < 1 || ny > g.hy || nseg < 1 || nseg > g.hz) return false;
+    if (units != 0 && units < 3) return false;
     p.nvg = nvg;
     p.ngrp = (nvec + nvg - 1) / nvg;
     if (p.ngrp > kColMaxGroups) return false;
@@ -84,7 +88,7 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
     if (g.hx > 128 || p.w.nb > 8) return false;
     p.units = (int)((kColMaxSmem - 128) / (p.recB + p.wB));
     if (p.units < 3) return false;
-    if (p.units > kColMaxUnits) p.units = kColMaxUnits;
+    p.units = std::min(p.units, units ? std::min(units, kColMaxUnits) : kColMaxUnits);
     p.smem = 128 + p.units * (p.recB + p.wB);
     const int64_t nt = (int64_t)p.ngrp * p.nyt * nseg * nblk;
     if (nt > 0x7fffffff) return false;
@@ -177,11 +181,8 @@ inline int col_plans(const SubGeom &g, int nblk, int nvec, int vby, int wb, int 
             for (int nseg = 1; nseg <= 4 && nseg * 4 <= g.hz; nseg *= 2)
                 for (int few = 0; few < 2; ++few) {
                     ColPlan p;
-                    if (!col_shape(g, nblk, nvec, vby, wb, nvg, ny, nseg, p)) continue;
-                    if (few) {  // three units: more CTAs per SM
-                        p.units = 3;
-                        p.smem = 128 + 3 * (p.recB + p.wB);
-                    }
+                    // few: three units, more CTAs per SM
+                    if (!col_shape(g, nblk, nvec, vby, wb, nvg, ny, nseg, few ? 3 : 0, p)) continue;
                     const double e = col_estimate(p, g, nblk, vby, wb, num_sms);
                     int at = n < most ? n++ : most - 1;
                     if (at == most - 1 && n == most && best[at].nvg && us[at] <= e) continue;
@@ -204,6 +205,12 @@ inline void col_tile_of(const ColPlan &p, int tile[3])
     tile[0] = p.nvg;
     tile[1] = 9;
     tile[2] = p.ny | p.nseg << 8 | p.units << 16;
+}
+
+// The shape of such an entry.  False: no fit.
+inline bool col_of_tile(const SubGeom &g, int nblk, int nvec, int vby, int wb, const int tile[3], ColPlan &out)
+{
+    return col_shape(g, nblk, nvec, vby, wb, tile[0], tile[2] & 255, std::max(1, (tile[2] >> 8) & 255), tile[2] >> 16, out);
 }
 
 // Row kernel parameters without a tune entry: tile[], returns the vectors per thread.

@@ -441,11 +441,7 @@ template <int VP, int WF> cudaError_t col_launch(const StepArgs &a)
     } else {
         if (!a.err || !a.alphaf) return cudaErrorNotSupported;
         ColPlan p{};
-        if (!col_shape(a.g, a.nblk, a.nvec, vfmt_bytes(VP), wfmt_bytes(WF), a.tile[0], a.tile[2] & 255,
-                       std::max(1, (a.tile[2] >> 8) & 255), p))
-            return cudaErrorNotSupported;
-        if (a.tile[2] >> 16) p.units = std::min(p.units, a.tile[2] >> 16);
-        p.smem = 128 + p.units * (p.recB + p.wB);
+        if (!col_of_tile(a.g, a.nblk, a.nvec, vfmt_bytes(VP), wfmt_bytes(WF), a.tile, p)) return cudaErrorNotSupported;
         const int64_t gstride = (int64_t)a.nblk * a.g.Ps * p.nvg * vfmt_bytes(VP);
         auto kern = a.active ? k_step_col<VP, WF, true> : k_step_col<VP, WF, false>;
         if constexpr (WF == W_F32_18) {

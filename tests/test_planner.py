@@ -1,0 +1,67 @@
+"""The planner's rules on the host (csrc/col_plan.h, no GPU): compiled with g++ behind a few C functions."""
+
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2301_05518_gb300", "csrc")
+
+GLUE = r"""
+#include "col_plan.h"
+using namespace tls;
+static SubGeom geom(const int *h) { return SubGeom{h[0], h[1], h[2], h[0] * h[1] * h[2], (h[0] * h[1] * h[2] + 31) / 32 * 32}; }
+static int out_of(const ColPlan &p, int *o)
+{
+    const int v[] = {p.nvg, p.ny, p.nseg, p.units, p.smem, p.ntile, p.threads};
+    for (int k = 0; k < 7; ++k) o[k] = v[k];
+    return 1;
+}
+extern "C" {
+int entry_shape(const int *h, int nblk, int nvec, int vby, int wb, const int *tile, int *o)
+{
+    ColPlan p;
+    return col_of_tile(geom(h), nblk, nvec, vby, wb, tile, p) ? out_of(p, o) : 0;
+}
+int best_shapes(const int *h, int nblk, int nvec, int vby, int wb, int most, int *tiles, int *o)
+{
+    ColPlan p[8] = {};
+    double us[8];
+    const int n = col_plans(geom(h), nblk, nvec, vby, wb, 152, p, us, most);
+    for (int k = 0; k < n; ++k) {
+        col_tile_of(p[k], tiles + 3 * k);
+        out_of(p[k], o + 7 * k);
+    }
+    return n;
+}
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "glue.cpp").write_text(GLUE)
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, "-o", str(d / "plan.so"),
+                           str(d / "glue.cpp")])
+    return ctypes.CDLL(str(d / "plan.so"))
+
+
+def ints(*v):
+    return (ctypes.c_int * len(v))(*v)
+
+
+def entry(plan, h, nvec, nvg, ny, nseg, units, vby=24, wb=72, nblk=8):
+    o = ints(*[0] * 7)
+    ok = plan.entry_shape(ints(*h), nblk, nvec, vby, wb, ints(nvg, 9, ny | nseg << 8 | units << 16), o)
+    return list(o) if ok else None
+
+
+@pytest.mark.parametrize("units,want", [(0, 6), (3, 3), (5, 5), (6, 6), (9, 6), (1, None), (2, None), (-1, None), (-3, None)])
+def test_ring_units_of_an_entry(plan, units, want):
+    """Fewer than three units are no ring: such a shape does not fit (the planner takes over)."""
+    got = entry(plan, (4, 4, 4), 8, 8, 2, 1, units)
+    assert (got and got[3]) == want
+    if got:
+        assert 0 < got[4] <= 226 * 1024
