@@ -72,6 +72,7 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
     ColPlan p{};
     if (nvg < 2 || (nvg & 1) || ny < 1 || ny > g.hy || nseg < 1 || nseg > g.hz) return false;
     if (units != 0 && units < 3) return false;
+    if (ny > 255) return false;  // a tune entry holds the rows in eight bits
     p.nvg = nvg;
     p.ngrp = (nvec + nvg - 1) / nvg;
     if (p.ngrp > kColMaxGroups) return false;

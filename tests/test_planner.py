@@ -65,3 +65,19 @@ def test_ring_units_of_an_entry(plan, units, want):
     assert (got and got[3]) == want
     if got:
         assert 0 < got[4] <= 226 * 1024
+
+
+@pytest.mark.parametrize("hy,hz,nblk,vby,wb", [(256, 4, 152, 24, 32), (256, 4, 1024, 24, 32), (256, 4, 152, 24, 24),
+                                               (480, 32, 304, 24, 24), (24, 24, 8, 24, 72), (17, 9, 40, 16, 24)])
+@pytest.mark.parametrize("nvec", [2, 4, 24])
+def test_planned_shape_is_the_launched_shape(plan, hy, hz, nblk, vby, wb, nvec):
+    """Shapes travel to the kernel as tune entries: what the planner chose is what the entry says, also
+    where a tile could take more rows than an entry can hold (2 x 512 x 8 sites a slice)."""
+    hx = 1 if hy > 100 else hy
+    tiles, o = ints(*[0] * 24), ints(*[0] * 56)
+    n = plan.best_shapes(ints(hx, hy, hz), nblk, nvec, vby, wb, 3, tiles, o)
+    assert n > 0
+    for k in range(n):
+        q = ints(*[0] * 7)
+        assert plan.entry_shape(ints(hx, hy, hz), nblk, nvec, vby, wb, ints(*tiles[3 * k:3 * k + 3]), q) == 1
+        assert list(q) == o[7 * k:7 * k + 7]
