@@ -826,24 +826,43 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         nslot = std::min(ngroup, 3);
         slot_bytes = (io_slice_bytes * tg * nvec + 255) / 256 * 256;
     }
-    auto workspace = [&]() -> tls_status {
+    auto buffers = [&](DevBuf *b[6], uint64_t need[6]) {
         const int last = (nvec - 1) / G * G;  // first vector of the last group
         nalpha = std::max(nvec + 1, last + packed_of(nvec - last));
         alpha_bytes = (sizeof(double) + sizeof(float)) * nalpha;
-        tls_status r = ensure(ctx, ctx->A, (size_t)vs * packed_of(G), "tls_smear: vector buffer A");
-        if (r == TLS_OK) r = ensure(ctx, ctx->B, (size_t)vs * packed_of(G), "tls_smear: vector buffer B");
-        if (r == TLS_OK) r = ensure(ctx, ctx->alpha, alpha_bytes, "tls_smear: alpha");
-        if (r == TLS_OK && norms_out)
-            r = ensure(ctx, ctx->partials, sizeof(double) * kNormPartsPerSlice * nsl * nvec, "tls_smear: partials");
-        if (r == TLS_OK && norms_out) r = ensure(ctx, ctx->norms, sizeof(double) * nvec, "tls_smear: norms");
-        if (r == TLS_OK && staged) r = ensure(ctx, ctx->staging, slot_bytes * nslot, "tls_smear: host staging");
+        DevBuf *const of[] = {&ctx->A, &ctx->B, &ctx->alpha, &ctx->partials, &ctx->norms, &ctx->staging};
+        const uint64_t n[] = {(size_t)vs * packed_of(G), (size_t)vs * packed_of(G), alpha_bytes,
+                              norms_out ? sizeof(double) * kNormPartsPerSlice * nsl * nvec : 0,
+                              norms_out ? sizeof(double) * nvec : 0, staged ? slot_bytes * nslot : 0};
+        std::copy(of, of + 6, b);
+        std::copy(n, n + 6, need);
+    };
+    auto workspace = [&]() -> tls_status {
+        static const char *const what[] = {"tls_smear: vector buffer A", "tls_smear: vector buffer B", "tls_smear: alpha",
+                                           "tls_smear: partials", "tls_smear: norms", "tls_smear: host staging"};
+        DevBuf *b[6];
+        uint64_t need[6];
+        buffers(b, need);
+        tls_status r = TLS_OK;
+        for (int k = 0; k < 6 && r == TLS_OK; ++k) r = ensure(ctx, *b[k], need[k], what[k]);
         return r;
     };
-    s = workspace();
-    if (s != TLS_OK && col && packed_of(G) > rec_of(G)) {  // once more without the padding of the vector groups
+    const bool padded = col && packed_of(G) > rec_of(G);
+    auto unpadded = [&] {  // without the padding of the vector groups
         col = false;
         vb = row_tile(g, nblk, col_n, VBY, tile);
         if (G0 % vb != 0) vb = default_il_vb(storage, G0);
+    };
+    if (padded) {
+        DevBuf *b[6];
+        uint64_t have[6], need[6];
+        buffers(b, need);
+        for (int k = 0; k < 6; ++k) have[k] = b[k]->n;
+        if (!workspace_fits(ctx->used.load(), ctx->cap, 6, have, need)) unpadded();
+    }
+    s = workspace();
+    if (s != TLS_OK && col && padded) {  // the device itself is full: once more
+        unpadded();
         release(ctx, ctx->A);
         release(ctx, ctx->B);
         s = workspace();

@@ -200,6 +200,16 @@ inline int col_plans(const SubGeom &g, int nblk, int nvec, int vby, int wb, int 
     return n;
 }
 
+// Whether buffers of have[k] bytes can grow to need[k] under an HBM cap (0: none) with `used` bytes
+// in use, the old ones counted.  Known before a buffer is given up: a call that tried the padded
+// groups of the column kernel and failed freed, allocated and cleared its buffers each time.
+inline bool workspace_fits(uint64_t used, uint64_t cap, int n, const uint64_t *have, const uint64_t *need)
+{
+    for (int k = 0; k < n; ++k)
+        if (need[k] > have[k]) used += need[k] - have[k];
+    return cap == 0 || used <= cap;
+}
+
 // tile[] of the tune entry for a shape: 9 selects the column kernel.
 inline void col_tile_of(const ColPlan &p, int tile[3])
 {

@@ -21,7 +21,7 @@ struct Cand {
     int tile[3];
 };
 
-std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, int num_sms)
+std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, int num_sms, bool exact)
 {
     // The kernels that won at some measured shape.  Measured and dropped (they
     // never won at any benchmarked shape): the register-capped and W-staged
@@ -37,7 +37,9 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
     if (storage != TLS_F64) {  // the column kernel at the tile shapes its cost model ranks first
         ColPlan best[3] = {};
         double us[3];
-        const int n = col_plans(gg.g, nsl * 8, G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms, best, us, 3);
+        // under an HBM cap only groups without padding, as the planner does
+        const int n = col_plans(gg.g, nsl * 8, exact ? (G + 1) & ~1 : G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms,
+                                best, us, 3, exact);
         if (nvec >= 2 && nvec <= 4 && gg.wfmt != W_F32_8)  // planar vectors in one launch
             c.push_back({TLS_KERNEL_MRHS, planar_vb(storage, nvec), 128, {0, 10, 0}});
         for (int k = 0; k < n; ++k) {
@@ -125,7 +127,7 @@ tls_status tls_autotune(tls_ctx *ctx, tls_gauge_id id, int nvec, int storage, in
     ctx->profiling = true;
     TuneVal win{0, 0, 0, {0, 0, 0}, 1e300};
     int n = 0;
-    for (const Cand &c : candidates(nvec, storage, gg, nsl, ctx->num_sms)) {
+    for (const Cand &c : candidates(nvec, storage, gg, nsl, ctx->num_sms, ctx->cap != 0)) {
         // one warm-up call, then the timed one
         s = smear_impl(ctx, id, tmp, io, 1, nvec, 1, 0.5, timeslice, storage, c.kernel, c.vb, c.threads, c.tile,
                        nullptr, nullptr);

@@ -35,6 +35,10 @@ int best_shapes(const int *h, int nblk, int nvec, int vby, int wb, int most, int
     }
     return n;
 }
+int fits(unsigned long long used, unsigned long long cap, int n, const unsigned long long *have, const unsigned long long *need)
+{
+    return workspace_fits(used, cap, n, (const uint64_t *)have, (const uint64_t *)need);
+}
 }
 """
 
@@ -81,3 +85,15 @@ def test_planned_shape_is_the_launched_shape(plan, hy, hz, nblk, vby, wb, nvec):
         q = ints(*[0] * 7)
         assert plan.entry_shape(ints(hx, hy, hz), nblk, nvec, vby, wb, ints(*tiles[3 * k:3 * k + 3]), q) == 1
         assert list(q) == o[7 * k:7 * k + 7]
+
+
+@pytest.mark.parametrize("used,cap,have,need,want", [
+    (100, 0, [0, 0], [1 << 40, 1 << 40], True),       # no cap
+    (100, 120, [40, 40], [50, 50], True),             # both grow by ten: 120 in use
+    (100, 119, [40, 40], [50, 50], False),
+    (100, 100, [40, 40], [40, 10], True),             # nothing grows, nothing shrinks
+    (100, 104, [40, 40], [10, 45], False),            # a buffer that is larger than needed stays
+    (100, 105, [40, 40], [10, 45], True)])
+def test_padding_is_decided_before_a_buffer_is_freed(plan, used, cap, have, need, want):
+    arr = ctypes.c_ulonglong * len(have)
+    assert bool(plan.fits(ctypes.c_ulonglong(used), ctypes.c_ulonglong(cap), len(have), arr(*have), arr(*need))) == want
