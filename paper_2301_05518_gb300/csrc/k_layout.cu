@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "layout_plan.h"
 #include "tls_dev.cuh"
 #include "tls_internal.h"
 
@@ -634,10 +635,10 @@ __global__ void __launch_bounds__(256) k_pack_rows(const IO *__restrict__ src, i
 // Pack and unpack of the FP32 and 16-bit interleaved records, by vector pairs.
 // A thread moves one record pair of one site: two canonical colour vectors of 24
 // (FP64 caller: 48) bytes each against one 16-byte word per colour, or one 32-byte
-// record.  CTA = one canonical x-row; consecutive lanes take the pairs of a site,
-// then the next site, so that the records of the even and of the odd sites of the
-// row are each written in one contiguous run (nvg = 8: 256 bytes per colour and
-// warp) and the canonical side is read in runs of a few sites per vector, every
+// record.  CTA = one or several canonical x-rows (pair_split); consecutive lanes take up
+// to four pairs of a site, then the next site, so that the records of the even and of the
+// odd sites of the row are written in runs (nvg = 8: contiguous, 256 bytes per colour and
+// warp) and the canonical side is read in runs of eight sites per vector, every
 // sector in full.  Both sides go straight between global memory and registers.
 // HBM-bound: 48^3 x 32, 24 vectors, FP32 1.00 / 1.33 ms (pack / unpack) with the
 // rows staged in shared memory one vector at a time, 0.58 / 0.82 now (4.1 GB moved); FP16
@@ -698,6 +699,7 @@ struct PairArgs {
     int nvec, rec_n, rec_v0;
     int64_t gstride;       // bytes between the fields of two groups
     bool rc, whole;        // rows contiguous; blocks are whole slices
+    PairSplit sp;
 };
 
 template <typename IO, int VP, bool PACK, bool AL>
@@ -705,18 +707,24 @@ __global__ void __launch_bounds__(256) k_move_pairs(std::conditional_t<PACK, con
                                                     std::conditional_t<PACK, char, const char> *__restrict__ recs,
                                                     SubGeom g, PairArgs a)
 {
-    const int y = blockIdx.x % a.Ly, z = blockIdx.x / a.Ly, ts = blockIdx.y;
+    const int ts = blockIdx.y;
     const int first = blockIdx.z * a.rec_n;  // vectors of the groups before this one
     const int nv = min(a.nvec - first, a.rec_n);
     const int u0 = a.rec_v0 >> 1, T = ((a.rec_v0 + nv + 1) >> 1) - u0;
-    const int sub0 = ((y & 1) << 1) | ((z & 1) << 2);
-    const int r = a.whole ? (z * g.hy + y) * g.hx : ((z >> 1) * g.hy + (y >> 1)) * g.hx;
-    const int64_t site0 = (((int64_t)(a.t_first + ts) * a.Lz + z) * a.Ly + y) * a.Lx;
     const int64_t sb = (int64_t)a.rec_n * VRec<VP>::SB;
     const int cs = (int)((a.rc ? g.hx : g.Ps) * a.rec_n);
-    const int64_t row = il_site<VP>(g, r, a.rc);
-    for (int k = threadIdx.x; k < T * a.Lx; k += blockDim.x) {
-        const int x = k / T, u = u0 + k - x * T;
+    const int C = a.sp.pairs, per = a.Lx * C, rowI = per * a.sp.chunks;
+    for (int k = threadIdx.x; k < a.sp.rows * rowI; k += blockDim.x) {
+        const int rl = k / rowI, j = k - rl * rowI;      // row, item of the row
+        const int ch = j / per, i = j - ch * per;        // chunk of pairs, item of the chunk
+        const int x = i / C, t = ch * C + i - x * C;     // site, pair
+        const int yz = blockIdx.x * a.sp.rows + rl;
+        if (t >= T || yz >= a.Ly * a.Lz) continue;
+        const int y = yz % a.Ly, z = yz / a.Ly, u = u0 + t;
+        const int sub0 = ((y & 1) << 1) | ((z & 1) << 2);
+        const int r = a.whole ? (z * g.hy + y) * g.hx : ((z >> 1) * g.hy + (y >> 1)) * g.hx;
+        const int64_t site0 = (((int64_t)(a.t_first + ts) * a.Lz + z) * a.Ly + y) * a.Lx;
+        const int64_t row = il_site<VP>(g, r, a.rc);
         const int v0 = 2 * u - a.rec_v0;
         const bool on0 = v0 >= 0, on1 = v0 + 1 < nv;
         const int b = a.whole ? ts : ts * 8 + (sub0 | (x & 1));
@@ -754,7 +762,7 @@ template <typename IO, bool PACK>
 cudaError_t move_pairs(const void *canon, char *recs, int prec, const SubGeom &g, int nsl, int ngrp, const PairArgs &a,
                        cudaStream_t s)
 {
-    const dim3 grid((unsigned)(a.Ly * a.Lz), nsl, ngrp);
+    const dim3 grid((unsigned)((a.Ly * a.Lz + a.sp.rows - 1) / a.sp.rows), nsl, ngrp);
     if (nsl > 65535 || ngrp > 65535) return cudaErrorInvalidConfiguration;
     const bool al = reinterpret_cast<uintptr_t>(canon) % (2 * sizeof(IO)) == 0;
     auto go = [&](auto k_al, auto k) {
@@ -957,8 +965,9 @@ static cudaError_t move_il(const void *canon, int io_prec, int64_t vs, char *rec
                    ? move_f64<double>(PACK, canon, vs, recs, g, L, t_first, nsl, nvec, rec_n, rec_v0, s)
                    : move_f64<float>(PACK, canon, vs, recs, g, L, t_first, nsl, nvec, rec_n, rec_v0, s);
     }
+    const int T = ((rec_v0 + std::min(nvec, rec_n) + 1) >> 1) - (rec_v0 >> 1);  // pairs of the largest group
     const PairArgs a{vs, L[0], L[1], L[2], t_first, nvec, rec_n, rec_v0, (int64_t)nsl * (whole ? 1 : 8) * g.Ps * rec_n * vfmt_bytes(prec),
-                     rc, whole};
+                     rc, whole, pair_split(T, L[0], L[1] * L[2])};
     return io_prec == P_F64 ? move_pairs<double, PACK>(canon, recs, prec, g, nsl, ngrp, a, s)
                             : move_pairs<float, PACK>(canon, recs, prec, g, nsl, ngrp, a, s);
 }

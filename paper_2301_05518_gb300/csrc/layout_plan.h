@@ -1,0 +1,33 @@
+// layout_plan.h -- how the kernels of k_layout.cu split their work.
+#pragma once
+
+#include <stdint.h>
+
+#include <algorithm>
+
+namespace tls {
+
+// Work of a CTA of 256 threads that moves vector pairs (k_move_pairs): `rows` canonical rows, each in
+// `chunks` chunks of `pairs` vector pairs; consecutive threads take the pairs of a chunk at one site,
+// then the next site.
+// At most four pairs a chunk: a warp then reads runs of eight sites of eight vectors.  With all
+// pairs of a site side by side it touched as many sectors as it has threads, and they had left
+// L1 before the next site used the rest of them (pack and unpack of 72 FP32 vectors, 12 x 36 x 36 x
+// 24: 1989 us with 36 pairs side by side, 735 with 12, 512 with 8, 494 with 4; 48^3 x 16: 10.6, 3.6,
+// 2.5 and 2.2 ms; 24 vectors there 981, 988, 767 and 731 us).  Several rows where one leaves
+// threads idle (4 x 48 x 48 x 24, 24 vectors in groups of eight: 211 us with one row, 125 with 16).
+struct PairSplit {
+    int rows, chunks, pairs;
+};
+
+// T pairs of rows of Lx sites, nrow rows a slice.
+inline PairSplit pair_split(int T, int Lx, int nrow)
+{
+    PairSplit p;
+    p.chunks = (T + 3) / 4;
+    p.pairs = (T + p.chunks - 1) / p.chunks;
+    p.rows = std::max(1, std::min(256 / (p.chunks * p.pairs * Lx), nrow));
+    return p;
+}
+
+}  // namespace tls

@@ -1,4 +1,4 @@
-"""The planner's rules on the host (csrc/col_plan.h, no GPU): compiled with g++ behind a few C functions."""
+"""The planner's rules on the host (csrc/col_plan.h, layout_plan.h; no GPU): compiled with g++ behind a few C functions."""
 
 import ctypes
 import os
@@ -10,6 +10,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 GLUE = r"""
 #include "col_plan.h"
+#include "layout_plan.h"
 using namespace tls;
 static SubGeom geom(const int *h) { return SubGeom{h[0], h[1], h[2], h[0] * h[1] * h[2], (h[0] * h[1] * h[2] + 31) / 32 * 32}; }
 static int out_of(const ColPlan &p, int *o)
@@ -34,6 +35,13 @@ int best_shapes(const int *h, int nblk, int nvec, int vby, int wb, int most, int
         out_of(p[k], o + 7 * k);
     }
     return n;
+}
+void split(int T, int Lx, int nrow, int *o)
+{
+    const PairSplit p = pair_split(T, Lx, nrow);
+    o[0] = p.rows;
+    o[1] = p.chunks;
+    o[2] = p.pairs;
 }
 int fits(unsigned long long used, unsigned long long cap, int n, const unsigned long long *have, const unsigned long long *need)
 {
@@ -97,3 +105,18 @@ def test_planned_shape_is_the_launched_shape(plan, hy, hz, nblk, vby, wb, nvec):
 def test_padding_is_decided_before_a_buffer_is_freed(plan, used, cap, have, need, want):
     arr = ctypes.c_ulonglong * len(have)
     assert bool(plan.fits(ctypes.c_ulonglong(used), ctypes.c_ulonglong(cap), len(have), arr(*have), arr(*need))) == want
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 4, 5, 9, 12, 13, 24, 36, 128])
+@pytest.mark.parametrize("Lx,nrow", [(2, 4), (4, 2304), (12, 1296), (48, 2304), (66, 6), (512, 4)])
+def test_pair_split_fills_the_threads(plan, T, Lx, nrow):
+    """Every pair has a place, at most four lie side by side, and a CTA of 256 threads is at least half
+    full unless the whole slice has less work or a chunk of another pair does not fit."""
+    p = ints(0, 0, 0)
+    plan.split(T, Lx, nrow, p)
+    rows, chunks, pairs = p
+    assert chunks * pairs >= T > (chunks - 1) * pairs and 1 <= pairs <= 4
+    assert 1 <= rows <= nrow
+    items = chunks * pairs * Lx
+    assert rows == 1 or rows * items <= 256
+    assert rows * items > 128 or rows == nrow
