@@ -493,44 +493,98 @@ __global__ void k_unpack_il(const char *__restrict__ src, IO *__restrict__ dst, 
     }
 }
 
-// Partial sums of |psi|^2 of canonical vectors, per (vector, slice, part): a cluster of
-// kNormSplit CTAs takes a fixed strided subset of the reals of slice s of vector v, so each
-// partial depends only on its own slice and the sum order is fixed.  Partial (v, s, p) goes to
-// partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].  Bound by the FP64 adds of
-// the SMs in use: with norms of one slice of 48^3, 3 vectors, a call takes 22 us longer, 38 with one
-// CTA per partial (and as long with 64 partials per slice, which take four times the scratch).
+// Partial sums of |psi|^2 of canonical vectors, per (vector, slice, part): part p of slice s of
+// vector v goes to partials[v * part_stride + part_off + s * kNormPartsPerSlice + p].  A part is
+// S strided subsets of the reals of its slice, 256 sums each, added up subset by subset and then as
+// a tree: S depends on the slice alone (norm_subsets), so a norm does not depend on the call
+// it is part of.  CL: a cluster of S CTAs, one subset each; otherwise one CTA takes all S, its sums
+// independent of one another.  The same bits.
+// Bound by the FP64 adds of the SMs in use.  With norms of one slice of 48^3, 3 vectors, a call
+// takes 22 us longer with clusters, 38 with one CTA per part; 24 FP32 vectors on 16 slices 1056 and
+// 998 us.  Small slices have one subset: a thread of four CTAs would have one or two reals and
+// the tree cost more than the sums (16^3 x 32, 72 vectors: 811 us with clusters, 269 now).
 constexpr int kNormSplit = 4;
-template <typename IO>
-__global__ void __cluster_dims__(kNormSplit, 1, 1) __launch_bounds__(256)
-    k_norm_partials(const IO *__restrict__ base, int64_t vstride, int64_t slice_sites, double *__restrict__ partials,
-                    int64_t part_stride, int64_t part_off)
+
+// v summed over the CTA in the order of a tree over the thread index; thread 0 has the sum.
+__device__ __forceinline__ double norm_tree(double v, double red[256])
 {
-    constexpr int kCtas = kNormPartsPerSlice * kNormSplit;  // of a slice
+    const int t = threadIdx.x;
+    red[t] = v;
+    __syncthreads();
+    if (t < 128) red[t] = v += red[t + 128];
+    __syncthreads();
+    if (t < 64) red[t] = v += red[t + 64];
+    __syncthreads();
+    if (t < 32) {
+        v += red[t + 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    }
+    return v;
+}
+
+template <typename IO, int S, bool CL>
+__device__ __forceinline__ void norm_partials(const IO *__restrict__ base, int64_t vstride, int64_t slice_sites,
+                                              double *__restrict__ partials, int64_t part_stride, int64_t part_off)
+{
+    constexpr int R = CL ? 1 : S;                            // subsets of this CTA
+    constexpr int kCtas = kNormPartsPerSlice * (CL ? S : 1);  // of a slice
     __shared__ double red[256];
     const int v = blockIdx.y;
     const int sl = blockIdx.x / kCtas, part = blockIdx.x - sl * kCtas;
     const IO *p = base + ((int64_t)v * vstride + (int64_t)sl * slice_sites) * 6;
     const int64_t n = slice_sites * 6;
-    double acc = 0.0;
-#pragma unroll 8
-    for (int64_t k = (int64_t)part * blockDim.x + threadIdx.x; k < n; k += (int64_t)kCtas * blockDim.x) {
-        const double x = (double)p[k];
-        acc = fma(x, x, acc);
+    constexpr int64_t step = (int64_t)kNormPartsPerSlice * S * 256;
+    double acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = 0.0;
+    int64_t k = (int64_t)part * R * 256 + threadIdx.x;
+#pragma unroll(R > 1 ? 2 : 8)
+    for (; k + (R - 1) * 256 < n; k += step)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double x = (double)p[k + r * 256];
+            acc[r] = fma(x, x, acc[r]);
+        }
+    if constexpr (R > 1) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (k + r * 256 < n) {
+                const double x = (double)p[k + r * 256];
+                acc[r] = fma(x, x, acc[r]);
+            }
     }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    double sum = acc[0];
+    if constexpr (CL) {
+        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        red[threadIdx.x] = sum;
+        cl.sync();
+        if (cl.block_rank() == 0)
+            for (int r = 1; r < S; ++r) sum += *cl.map_shared_rank(red + threadIdx.x, r);
+        cl.sync();  // no CTA leaves or reuses its sums while they are read
+        if (cl.block_rank() != 0) return;
+    } else {
+#pragma unroll
+        for (int r = 1; r < R; ++r) sum += acc[r];
     }
-    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-    cl.sync();
-    if (cl.block_rank() == 0 && threadIdx.x == 0) {
-        double sum = red[0];
-        for (int r = 1; r < kNormSplit; ++r) sum += *cl.map_shared_rank(red, r);
-        partials[(int64_t)v * part_stride + part_off + blockIdx.x / kNormSplit] = sum;
-    }
-    cl.sync();  // no CTA leaves while its sum is read
+    sum = norm_tree(sum, red);
+    if (threadIdx.x == 0) partials[(int64_t)v * part_stride + part_off + blockIdx.x / (CL ? S : 1)] = sum;
+}
+
+template <typename IO, int S>
+__global__ void __launch_bounds__(256)
+    k_norm_partials(const IO *__restrict__ base, int64_t vstride, int64_t slice_sites, double *__restrict__ partials,
+                    int64_t part_stride, int64_t part_off)
+{
+    norm_partials<IO, S, false>(base, vstride, slice_sites, partials, part_stride, part_off);
+}
+
+template <typename IO>
+__global__ void __cluster_dims__(kNormSplit, 1, 1) __launch_bounds__(256)
+    k_norm_partials_cl(const IO *__restrict__ base, int64_t vstride, int64_t slice_sites, double *__restrict__ partials,
+                       int64_t part_stride, int64_t part_off)
+{
+    norm_partials<IO, kNormSplit, true>(base, vstride, slice_sites, partials, part_stride, part_off);
 }
 
 // Copies the interleaved records of one x'-row (hx sites starting at site r of
@@ -987,21 +1041,31 @@ cudaError_t launch_unpack_il(const char *src, int prec, void *dst, int io_prec, 
                           rec_v0, s, rc, whole);
 }
 
+template <typename IO>
+static cudaError_t norm_launch(const void *base, int64_t vstride_sites, int64_t slice_sites, int nsl, int nvec,
+                               double *partials, int64_t part_stride, int64_t part_off, cudaStream_t s)
+{
+    const IO *p = (const IO *)base;
+    const dim3 one(nsl * kNormPartsPerSlice, nvec), split(nsl * kNormPartsPerSlice * kNormSplit, nvec);
+    if (norm_subsets(slice_sites, kNormSplit) == 1)
+        k_norm_partials<IO, 1><<<one, 256, 0, s>>>(p, vstride_sites, slice_sites, partials, part_stride, part_off);
+    else if (norm_cluster(nsl, nvec))
+        k_norm_partials_cl<IO><<<split, 256, 0, s>>>(p, vstride_sites, slice_sites, partials, part_stride, part_off);
+    else
+        k_norm_partials<IO, kNormSplit><<<one, 256, 0, s>>>(p, vstride_sites, slice_sites, partials, part_stride, part_off);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_norm_partials(const void *base, int io_prec, int64_t vstride_sites, int64_t slice_sites, int nsl,
                                  int nvec, double *partials, int64_t part_stride, int64_t part_off, cudaStream_t s)
 {
     if (nvec == 0 || nsl == 0) return cudaSuccess;
     if ((int64_t)nsl * kNormPartsPerSlice * kNormSplit > 0x7fffffff || nvec > 65535) return cudaErrorInvalidValue;
-    dim3 grid(nsl * kNormPartsPerSlice * kNormSplit, nvec);
     if (io_prec == P_F64)
-        k_norm_partials<double><<<grid, 256, 0, s>>>((const double *)base, vstride_sites, slice_sites, partials,
-                                                      part_stride, part_off);
-    else if (io_prec == P_F32)
-        k_norm_partials<float><<<grid, 256, 0, s>>>((const float *)base, vstride_sites, slice_sites, partials,
-                                                     part_stride, part_off);
-    else
-        return cudaErrorNotSupported;
-    return cudaGetLastError();
+        return norm_launch<double>(base, vstride_sites, slice_sites, nsl, nvec, partials, part_stride, part_off, s);
+    if (io_prec == P_F32)
+        return norm_launch<float>(base, vstride_sites, slice_sites, nsl, nvec, partials, part_stride, part_off, s);
+    return cudaErrorNotSupported;
 }
 
 cudaError_t launch_reduce_norms(const double *partials, int nparts, int nvec, double *norms, cudaStream_t s)

@@ -30,4 +30,12 @@ inline PairSplit pair_split(int T, int Lx, int nrow)
     return p;
 }
 
+// Strided subsets of a part of a slice's norm, `split` or one: by the slice alone, since it sets the
+// order of the additions.  From 28^3 sites on a thread of `split` CTAs has eight reals or more.
+inline int norm_subsets(int64_t slice_sites, int split) { return slice_sites * 6 >= 131072 ? split : 1; }
+
+// Whether the subsets of a part are spread over a cluster: where one CTA per part (16 per slice
+// and vector) leaves SMs idle.  The sums are the same either way.
+inline bool norm_cluster(int nsl, int nvec) { return (int64_t)nsl * nvec * 16 < 8 * 152; }
+
 }  // namespace tls
