@@ -63,11 +63,14 @@ struct ColPlan {
     ColW w;
 };
 
+inline int col_smem(const ColPlan &p) { return 128 + p.units * (p.recB + p.wB); }
+
 // The tile shape: nvg vectors per group, ny rows, nseg segments, at most `units` ring units (0: as
 // many as fit).  False: no fit.  Fewer than three units are no ring: a consumer keeps the unit
 // before the one it waits for, and the producer runs one further.
+// w: col_w_plan of the tile's rows, if the caller has it.
 inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int nvg, int ny, int nseg, int units,
-                      ColPlan &out)
+                      ColPlan &out, const ColW *w = nullptr)
 {
     ColPlan p{};
     if (nvg < 2 || (nvg & 1) || ny < 1 || ny > g.hy || nseg < 1 || nseg > g.hz) return false;
@@ -84,13 +87,13 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
     p.threads = (int)((act + 31) / 32 * 32);
     const int64_t recB = (int64_t)(p.ny + 2) * g.hx * nvg * vby;
     p.recB = (int)((recB + 127) / 128 * 128);
-    p.w = col_w_plan(wb, g.hx, p.ny);
+    p.w = w ? *w : col_w_plan(wb, g.hx, p.ny);
     p.wB = p.w.bytes;
     if (g.hx > 128 || p.w.nb > 8) return false;
     p.units = (int)((kColMaxSmem - 128) / (p.recB + p.wB));
     if (p.units < 3) return false;
     p.units = std::min(p.units, units ? std::min(units, kColMaxUnits) : kColMaxUnits);
-    p.smem = 128 + p.units * (p.recB + p.wB);
+    p.smem = col_smem(p);
     const int64_t nt = (int64_t)p.ngrp * p.nyt * nseg * nblk;
     if (nt > 0x7fffffff) return false;
     p.ntile = (int)nt;
@@ -107,8 +110,9 @@ inline bool col_shape(const SubGeom &g, int nblk, int nvec, int vby, int wb, int
 // a copy's latency of 2350 cycles plus its transfer.  A tile of n planes takes n + 2
 // units; the whole cannot beat the memory.  A thread rebuilds W for one vector pair
 // only, so W formats that need arithmetic cost it more than the row kernel; groups of
-// two or four vectors measured about an eighth above the fit.
-inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby, int wb, int num_sms)
+// two or four vectors measured about an eighth above the fit.  A shape that its largest term alone
+// puts at `limit` or above gets that as its estimate.
+inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby, int wb, int num_sms, double limit)
 {
     const int warps = p.threads / 32;
     int occ = 1;
@@ -119,10 +123,13 @@ inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby
     const double unit = p.recB + p.wB;
     const double comp = (356 + 650.0 * ((warps * eff + 3) / 4)) * (vby == 16 ? 1.145 : 1.0) * fmt;
     const double copy = eff * unit / 36.5, lat = (2350 + unit / 36.5) / (p.units - 2);
-    const double t = std::pow(std::pow(comp, 6) + std::pow(copy, 6) + std::pow(lat, 6), 1.0 / 6);
-    const double us = rounds * ((double)g.hz / p.nseg + 2) * t / 2060;
     const double dram = (double)nblk * g.Vs * (3.0 * wb + 2.0 * vby * p.ngrp * p.nvg) / 6.4e6;
-    return std::max(us, dram) * (1 + (rounds > 1 ? 0.005 : 0.03) * (p.units - 3)) + 3.5;
+    const double units = 1 + (rounds > 1 ? 0.005 : 0.03) * (p.units - 3);
+    auto total = [&](double t) { return std::max(rounds * ((double)g.hz / p.nseg + 2) * t / 2060, dram) * units + 3.5; };
+    const double low = total(std::max(std::max(comp, copy), lat));
+    if (low >= limit) return low;
+    auto p6 = [](double x) { return x * x * x * x * x * x; };
+    return total(std::cbrt(std::sqrt(p6(comp) + p6(copy) + p6(lat))));
 }
 
 // The same for the row kernel (k_ilt.cuh): 0.03 + 0.0105 n ns per site for n vectors
@@ -168,33 +175,45 @@ inline double planar_estimate(const SubGeom &g, int nblk, int nvec, int vby, int
 
 // The best tile shapes by that estimate, best first (at most `most`).  nvg divides
 // the vectors into equal groups with at most a third of padding (exact: none).
+// Runs in every call without a tune entry, before anything is enqueued: what a shape shares with
+// others is worked out once and most shapes are dropped by the largest term of their estimate
+// (48^3, one slice, 24 vectors 40 -> 5 us on an x86 host; 4 x 48 x 48, 72 vectors 103 -> 13).
 inline int col_plans(const SubGeom &g, int nblk, int nvec, int vby, int wb, int num_sms, ColPlan *best, double *us,
                      int most, bool exact = false)
 {
     int n = 0;
     const int n2 = (nvec + 1) & ~1;
-    for (int nvg = 2; nvg <= 24 && nvg <= n2; nvg += 2) {
-        if ((nvec + nvg - 1) / nvg * nvg * 3 > 4 * n2 || (exact && nvec % nvg)) continue;
-        for (int last = 0, nyt = 1; nyt <= g.hy; ++nyt) {
-            const int ny = (g.hy + nyt - 1) / nyt;
-            if (ny == last) continue;
-            last = ny;
-            for (int nseg = 1; nseg <= 4 && nseg * 4 <= g.hz; nseg *= 2)
-                for (int few = 0; few < 2; ++few) {
-                    ColPlan p;
-                    // few: three units, more CTAs per SM
-                    if (!col_shape(g, nblk, nvec, vby, wb, nvg, ny, nseg, few ? 3 : 0, p)) continue;
-                    const double e = col_estimate(p, g, nblk, vby, wb, num_sms);
+    for (int last = 0, nyt = 1; nyt <= g.hy; ++nyt) {
+        const int ny = (g.hy + nyt - 1) / nyt;
+        if (ny == last) continue;
+        last = ny;
+        if ((int64_t)ny * g.hx > kColMaxThreads - 32) continue;
+        const ColW w = col_w_plan(wb, g.hx, ny);
+        for (int nvg = 2; nvg <= 24 && nvg <= n2; nvg += 2) {
+            if ((nvec + nvg - 1) / nvg * nvg * 3 > 4 * n2 || (exact && nvec % nvg)) continue;
+            ColPlan p;
+            if (!col_shape(g, nblk, nvec, vby, wb, nvg, ny, 1, 0, p, &w)) continue;
+            const int most_units = p.units, tiles = p.ntile;
+            for (int nseg = 1; nseg <= 4 && nseg * 4 <= g.hz; nseg *= 2) {
+                if ((int64_t)tiles * nseg > 0x7fffffff) break;
+                p.nseg = nseg;
+                p.ntile = tiles * nseg;
+                for (int units : {most_units, 3}) {  // three: more CTAs per SM
+                    p.units = units;
+                    p.smem = col_smem(p);
+                    const double limit = n < most ? 1e300 : us[n - 1];
+                    const double e = col_estimate(p, g, nblk, vby, wb, num_sms, limit);
+                    if (n == most && e >= limit) continue;
                     int at = n < most ? n++ : most - 1;
-                    if (at == most - 1 && n == most && best[at].nvg && us[at] <= e) continue;
-                    while (at > 0 && us[at - 1] > e) {
+                    for (; at > 0 && us[at - 1] > e; --at) {
                         best[at] = best[at - 1];
                         us[at] = us[at - 1];
-                        --at;
                     }
                     best[at] = p;
                     us[at] = e;
+                    if (most_units == 3) break;
                 }
+            }
         }
     }
     return n;

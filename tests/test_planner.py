@@ -36,6 +36,11 @@ int best_shapes(const int *h, int nblk, int nvec, int vby, int wb, int most, int
     }
     return n;
 }
+double estimate(const int *h, int nblk, int nvec, int vby, int wb, const int *tile)
+{
+    ColPlan p;
+    return col_of_tile(geom(h), nblk, nvec, vby, wb, tile, p) ? col_estimate(p, geom(h), nblk, vby, wb, 152, 1e300) : 1e300;
+}
 void split(int T, int Lx, int nrow, int *o)
 {
     const PairSplit p = pair_split(T, Lx, nrow);
@@ -57,7 +62,9 @@ def plan(tmp_path_factory):
     (d / "glue.cpp").write_text(GLUE)
     subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, "-o", str(d / "plan.so"),
                            str(d / "glue.cpp")])
-    return ctypes.CDLL(str(d / "plan.so"))
+    lib = ctypes.CDLL(str(d / "plan.so"))
+    lib.estimate.restype = ctypes.c_double
+    return lib
 
 
 def ints(*v):
@@ -120,3 +127,29 @@ def test_pair_split_fills_the_threads(plan, T, Lx, nrow):
     items = chunks * pairs * Lx
     assert rows == 1 or rows * items <= 256
     assert rows * items > 128 or rows == nrow
+
+
+@pytest.mark.parametrize("h,nblk,nvec", [((24, 24, 24), 8, 24), ((24, 24, 24), 256, 72), ((2, 24, 24), 8, 72), ((5, 17, 3), 40, 7),
+                                         ((1, 9, 8), 512, 3), ((33, 4, 16), 8, 30), ((8, 64, 64), 1, 12)])
+@pytest.mark.parametrize("vby,wb", [(24, 72), (16, 24)])
+def test_search_finds_the_best_shapes(plan, h, nblk, nvec, vby, wb):
+    """Shapes dropped early by a lower bound are none of the best three: against the full list, each shape
+    estimated without a limit."""
+    every = set()
+    for nvg in range(2, 26, 2):
+        if -(-nvec // nvg) * nvg * 3 > 4 * ((nvec + 1) & ~1) or nvg > ((nvec + 1) & ~1):
+            continue
+        for ny in {-(-h[1] // t) for t in range(1, h[1] + 1)}:
+            for nseg in (1, 2, 4):
+                if nseg * 4 <= h[2]:
+                    for units in (0, 3):
+                        got = entry(plan, h, nvec, nvg, ny, nseg, units, vby, wb, nblk)
+                        if got:
+                            every.add((got[0], 9, got[1] | got[2] << 8 | got[3] << 16))
+    times = sorted(plan.estimate(ints(*h), nblk, nvec, vby, wb, ints(*t)) for t in every)
+    tiles, o = ints(*[0] * 24), ints(*[0] * 56)
+    n = plan.best_shapes(ints(*h), nblk, nvec, vby, wb, 3, tiles, o)
+    assert n == min(3, len(times))
+    for k in range(n):
+        t = tuple(tiles[3 * k:3 * k + 3])
+        assert t in every and plan.estimate(ints(*h), nblk, nvec, vby, wb, ints(*t)) == times[k]
