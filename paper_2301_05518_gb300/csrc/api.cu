@@ -741,25 +741,32 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         col = col_of_tile(g, nblk, col_n, VBY, wfmt_bytes(fmt), tile, cp);
         planned = !col;
     }
-    if (col_ok && planned) {
-        double us = 0;
-        const double row_us = row_estimate(g, nblk, col_n, VBY, wfmt_bytes(fmt));
-        // under an HBM cap only groups without padding: buffers stay as large as the row kernel's
-        const bool exact = ctx->cap != 0;
-        const bool have_col =
-            col_plans(g, nblk, exact ? (col_n + 1) & ~1 : col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, &cp, &us, 1, exact) > 0;
-        if (op == 0 && planar_ok(g, nblk, nvec, wfmt_bytes(fmt)) &&
-            planar_estimate(g, nblk, nvec, VBY, wfmt_bytes(fmt)) < (have_col ? std::min(us, row_us) : row_us)) {
-            tile[1] = 10;
-        } else if (have_col && us < row_us) {
-            col = true;
-            vb = 2;
-            col_tile_of(cp, tile);
-        } else {
-            vb = row_tile(g, nblk, col_n, VBY, tile);
-            threads = 0;
+    // Host vectors go through slice groups of about kGroupBytes in up to three
+    // rotating staging slots, so that copies in and out overlap the smearing
+    // of other groups.  The persistent kernel takes all slices in one group.
+    const bool staged = !vecs_on_device;
+    int tg = nsl, ngroup = 1, nslot = 1;
+    size_t slot_bytes = 0;
+    if (staged) {
+        const size_t total = io_slice_bytes * nsl * nvec;
+        if (kern != TLS_KERNEL_PERSISTENT && nsl >= 2) {
+            const int64_t want = std::max<int64_t>(4, (int64_t)((total + kGroupBytes - 1) / kGroupBytes));
+            tg = (int)((nsl + std::min<int64_t>(nsl, want) - 1) / std::min<int64_t>(nsl, want));
+            ngroup = (nsl + tg - 1) / tg;
         }
+        nslot = std::min(ngroup, 3);
+        slot_bytes = (io_slice_bytes * tg * nvec + 255) / 256 * 256;
     }
+    auto plan = [&](bool exact) {  // for the slices of one launch
+        const StepPlan p = plan_step(g, tg * bps, nvec, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, exact, op == 0);
+        col = p.kind == STEP_COL;
+        cp = p.col;
+        vb = p.vb;
+        threads = 0;
+        for (int k = 0; k < 3; ++k) tile[k] = p.tile[k];
+    };
+    // under an HBM cap only groups without padding: buffers stay as large as the row kernel's
+    if (col_ok && planned) plan(ctx->cap != 0);
     // FP32 and 16-bit records of the interleaved layout come in vector pairs:
     // a group of an odd number of vectors carries one padding record
     // (computed, never unpacked).
@@ -788,20 +795,24 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     }
     // The multi-RHS kernel works on the interleaved layout in groups of <= 256 vectors.
     // tile[1] = 10: planar vectors, all of them in one launch (few vectors)
-    const bool planar = kern == TLS_KERNEL_MRHS && op == 0 && tile[1] == 10 && nvec <= 8;
-    if (planar) {
-        vb = planar_vb(storage, nvec);
-        threads = 128;
-    }
-    const bool il_layout = !planar && (kern == TLS_KERNEL_MRHS || kern == TLS_KERNEL_MRHS_ROWS || kern == TLS_KERNEL_MRHS_ZM);
-    const int G = il_layout ? std::min(nvec, gmax) : nvec;
+    bool planar = false, il_layout = false;
+    int G = nvec;
+    auto set_planar = [&] {
+        planar = kern == TLS_KERNEL_MRHS && op == 0 && tile[1] == 10 && nvec <= 8;
+        if (planar) {
+            vb = planar_vb(storage, nvec);
+            threads = 128;
+        }
+        il_layout = !planar && (kern == TLS_KERNEL_MRHS || kern == TLS_KERNEL_MRHS_ROWS || kern == TLS_KERNEL_MRHS_ZM);
+        G = il_layout ? std::min(nvec, gmax) : nvec;
+    };
+    set_planar();
 
     // Host vectors go through bulk copies (DMA) into a staging buffer.  On a
     // GB300 these measured faster than letting the layout kernels read and
     // write pinned host memory over NVLink-C2C directly (1236 ms against
     // 1436-1450 ms for the 64^3x96 step), so zero-copy is not used.
     void *vecs_dev = vecs_on_device ? vecs : nullptr;
-    const bool staged = vecs_dev == nullptr;
 
     // Workspace.
     auto packed_of = [&](int n) {  // records per site in the packed buffers
@@ -811,21 +822,6 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     // kernels); entries for the padding records of the last group too
     int nalpha = 0;
     size_t alpha_bytes = 0;
-    // Host vectors go through slice groups of about kGroupBytes in up to three
-    // rotating staging slots, so that copies in and out overlap the smearing
-    // of other groups.  The persistent kernel takes all slices in one group.
-    int tg = nsl, ngroup = 1, nslot = 1;
-    size_t slot_bytes = 0;
-    if (staged) {
-        const size_t total = io_slice_bytes * nsl * nvec;
-        if (kern != TLS_KERNEL_PERSISTENT && nsl >= 2) {
-            const int64_t want = std::max<int64_t>(4, (int64_t)((total + kGroupBytes - 1) / kGroupBytes));
-            tg = (int)((nsl + std::min<int64_t>(nsl, want) - 1) / std::min<int64_t>(nsl, want));
-            ngroup = (nsl + tg - 1) / tg;
-        }
-        nslot = std::min(ngroup, 3);
-        slot_bytes = (io_slice_bytes * tg * nvec + 255) / 256 * 256;
-    }
     auto buffers = [&](DevBuf *b[6], uint64_t need[6]) {
         const int last = (nvec - 1) / G * G;  // first vector of the last group
         nalpha = std::max(nvec + 1, last + packed_of(nvec - last));
@@ -849,9 +845,10 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     };
     const bool padded = col && packed_of(G) > rec_of(G);
     auto unpadded = [&] {  // without the padding of the vector groups
-        col = false;
-        vb = row_tile(g, nblk, col_n, VBY, tile);
-        if (G0 % vb != 0) vb = default_il_vb(storage, G0);
+        plan(true);
+        if (vb <= 0 || G0 % vb != 0) vb = default_il_vb(storage, G0);
+        if (threads == 0) threads = 256;
+        set_planar();
     };
     if (padded) {
         DevBuf *b[6];

@@ -132,45 +132,138 @@ inline double col_estimate(const ColPlan &p, const SubGeom &g, int nblk, int vby
     return total(std::cbrt(std::sqrt(p6(comp) + p6(copy) + p6(lat))));
 }
 
-// The same for the row kernel (k_ilt.cuh): 0.03 + 0.0105 n ns per site for n vectors
-// in fours (0.0125 n above 24, 0.0165 n where a row's vectors take several CTAs), 0.02 +
-// 0.015 n otherwise (48^3 x 32: 3 / 5 / 12 / 24 / 72 vectors 224 / 394 / 578 / 1018 / 3510
-// us; 64^3 x 24: 8 / 24 vectors 595 / 1624 us; rows of 48, 24 vectors 0.0170 n), 1.75 times that where its TMA copies do not apply (50^3 x 16, 24 vectors: 884
-// us), with the arithmetic of the W formats shared by four vectors (24 vectors at
-// 48^3 x 32, row / column kernel: f32-18 1018 / 927, f32-12 1103 / 1065, f32-8 1699 /
-// above 2600, 16-bit vectors with f32-18 1203 / 1037, with f16-12 1393 / 1414 us).
-// Rows (CTAs of the row kernel): one starts about every nanosecond (16^3 x 32: 16384 of them,
-// 17.7 us per step with 3 vectors).
-inline double row_ctas(const SubGeom &g, int nblk) { return (double)nblk * g.hy * g.hz; }
+// Sites per CTA for the interleaved kernels: nvec * spb <= threads, with a
+// whole number of warps when possible.
+inline int il_spb(int nvec, int threads)
+{
+    if (threads <= 0) threads = 256;
+    int spb = std::max(1, threads / nvec);
+    for (int s = spb; s >= 1; --s)
+        if ((s * nvec) % 32 == 0) return s;
+    return spb;
+}
 
-inline double row_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb)
+// Shared-memory bytes of a CTA of the row kernel: the mbarrier (128 bytes) and the five W rows.
+inline int row_smem(int hx, int wb) { return 128 + 5 * hx * wb; }
+constexpr int kRowMaxSmem = 48 << 10;
+
+// Whether its TMA staging applies: every plane segment of a W row starts and ends on a
+// 16-byte boundary (the remainder plane has 4 or 8 bytes per site).
+inline bool row_tma(int hx, int wb) { return (hx * (wb % 16)) % 16 == 0; }
+
+// Vectors per CTA of the row kernel: `want` if it is a multiple of vb dividing nvec, else the
+// largest such count with (count / vb) * hx <= 256 threads.  0: no fit.
+inline int row_group(int nvec, int vb, int hx, int want)
+{
+    auto fits = [&](int n) { return n >= vb && n % vb == 0 && nvec % n == 0 && (n / vb) * hx <= 256; };
+    if (want > 0 && fits(want)) return want;
+    for (int n = nvec; n >= vb; n -= vb)
+        if (fits(n)) return n;
+    return 0;
+}
+
+// Estimated time of one step (us) of the other kernels, fitted to 1600 measured (lattice, slices,
+// vectors, storage, W format) problems on a GB300: cubes of 8 to 64 and boxes of 4 to 64, even and odd
+// rows, 1 to 64 slices, 2 to 96 vectors.  Each is a latency of the step and, per warp of
+// an SM, a time that depends on the formats (us; two and four vectors a thread), beside
+// the bytes at 6.6 TB/s and what a CTA costs by itself.  Spread of estimate / measurement:
+// 10 % for the interleaved kernels, 13 % for the row and the planar one.
+enum StepFmt { SF_32_18, SF_32_12, SF_32_8, SF_32_18_H, SF_16_18, SF_16_12, SF_N };  // W (_H: 16-bit vectors)
+
+inline int step_fmt(int vby, int wb)
+{
+    switch (wb) {
+    case 72: return vby == 16 ? SF_32_18_H : SF_32_18;
+    case 48: return SF_32_12;
+    case 32: return SF_32_8;
+    case 36: return SF_16_18;
+    default: return SF_16_12;
+    }
+}
+
+inline double step_bytes(const SubGeom &g, int nblk, int n, int vby, int wb)
+{
+    return (double)nblk * g.Vs * (3.0 * wb + 2.0 * vby * n);
+}
+
+// Plain interleaved kernel (k_step_il), n vectors (an even number): any row, no staging.
+inline double il_estimate(const SubGeom &g, int nblk, int n, int vby, int wb, int num_sms)
+{
+    static const double per_warp[SF_N][2] = {{.109, .252}, {.092, .198}, {.202, .324}, {.105, .269}, {.109, .235}, {.129, .225}};
+    const int vb = n % 4 ? 2 : 4, tx = n / vb, spb = std::max(1, std::min(il_spb(tx, 256), g.hx));
+    const double warps = (double)((g.hx + spb - 1) / spb) * g.hy * g.hz * nblk * ((tx * spb + 31) / 32);
+    return 5.2 + (wb == 32 ? 2.0 : 0.0) + step_bytes(g, nblk, n, vby, wb) / 9.0e6 +
+           per_warp[step_fmt(vby, wb)][vb / 4] * warps / num_sms;
+}
+
+// Row kernel parameters without a tune entry: tile[], returns the vectors per thread.
+// More than 24 vectors go through CTAs of 24 where that divides them (72 vectors at
+// 48^3 x 24: 2.41 ms against 2.64 with 36 a CTA); rows are asked into L2 ahead (tile[2])
+// where a step's data do not stay there (64^3 x 24, 24 vectors: 1.61 against 1.64 ms;
+// 16^3 x 32, 2 vectors: 21 against 19 us).  Four vectors per thread where the rows then still
+// fill a warp (32^3 x 64 / 48^3 x 32, 3 vectors: 16 / 24 threads, 180 / 224 us with four and
+// 142 / 290 with two); 16-bit records want twice the threads (12 vectors, 48 threads: 434
+// against 369 us; 24 vectors, 144 threads: 1203 against 1507).
+inline int row_tile(const SubGeom &g, int nblk, int nvec, int vby, int tile[3])
 {
     const int n = (nvec + 1) & ~1;
-    const double fmt = wb == 48 ? 1.08 : wb == 32 ? 1.65 : wb == 24 ? 1.15 : 1.0;
-    const bool split = n / 4 * g.hx > 256;  // the vectors of a row take several CTAs
-    const double site = n % 4 ? 0.02 + 0.015 * n : split ? 0.0165 * n : n > 24 ? 0.0125 * n : 0.03 + 0.0105 * n;
-    const bool tma = (g.hx * (wb % 16)) % 16 == 0;
-    const double us = (double)nblk * g.Vs * site * 1e-3 * (tma ? 1.0 : 1.75) * (vby == 16 ? 1.2 : 1.0) * fmt;
-    return std::max(us, row_ctas(g, nblk) * 1e-3) + 2;
+    tile[0] = n > 24 && n % 24 == 0 ? 24 : 0;
+    tile[1] = 6;
+    tile[2] = (double)nblk * g.Vs * (216.0 + 2.0 * vby * n) > 120e6 ? -1 : 0;
+    return n % 4 == 0 && n / 4 * g.hx >= (vby == 16 ? 64 : 20) ? 4 : 2;
 }
 
-// All vectors in one launch of the planar kernel, two or four a thread: reads W once, has
-// no rows to keep whole, but pays for unused lanes of its four vectors (16^3 x 32, 2 / 3 / 4
-// vectors: 7.0 / 11.3 / 13.9 us per step against 12.1 / 17.7 / 17.7; 48^3 x 32: 202 / 375 /
-// 460 against 186 / 231 / 231; 32^3 x 16, 2 FP16 vectors with W f16-12: 27 against 47).
-// A candidate for two vectors, and for up to four where the row kernel is bound by starting
-// its CTAs.  Not for the 8-real W, whose reconstruction rounds differently there.
-inline bool planar_ok(const SubGeom &g, int nblk, int nvec, int wb)
+// Row kernel with the parameters of row_tile; where its copies do not apply, the packed kernel
+// (k_step_ilx) that runs instead.  Where the vectors of a row do not divide, a CTA is left with one
+// pair or two and copies the five W rows for them: no candidate then (44^3, one slice, 26
+// vectors with W f32-12: 103 us against 51 with the interleaved kernel).
+inline double row_estimate(const SubGeom &g, int nblk, int n, int vby, int wb, int num_sms)
 {
-    return wb != 32 && (nvec == 2 || (nvec > 2 && nvec <= 4 && row_ctas(g, nblk) > 8000));
+    static const double per_warp[SF_N][2] = {{.145, .223}, {.149, .233}, {.254, .358}, {.148, .255}, {.161, .284}, {.171, .291}};
+    static const double packed[SF_N][2] = {{.028, .042}, {.05, .08}, {.2, .3}, {.071, .150}, {.089, .155}, {.093, .185}};
+    int tile[3];
+    const int vb = row_tile(g, nblk, n, vby, tile), f = step_fmt(vby, wb);
+    const double rows = (double)nblk * g.hy * g.hz;
+    const int nvg = row_group(n, vb, g.hx, tile[0]);
+    if (row_tma(g.hx, wb) && nvg > 0 && row_smem(g.hx, wb) <= kRowMaxSmem) {
+        if (nvg < 8 && nvg < n) return 1e300;
+        const double ctas = rows * (n / nvg);
+        const double a = per_warp[f][vb / 4] * ctas * ((nvg / vb * g.hx + 31) / 32) / num_sms;
+        const double b = 1.3e-4 * ctas, w = 0.116e-6 * ctas * g.hx * 5 * wb;  // starting them; their W rows from L2
+        return (wb == 32 ? 4.0 : 2.3) + std::sqrt(a * a + b * b + w * w);
+    }
+    const int tx = n / vb, spb = std::max(1, std::min(std::min(il_spb(tx, 256), g.hx), 56));
+    const double ctas = rows * ((g.hx + spb - 1) / spb);
+    return 5.4 + step_bytes(g, nblk, n, vby, wb) / 3.5e6 + 7.2e-4 * ctas +
+           packed[f][vb / 4] * ctas * ((tx * spb + 31) / 32) / num_sms;
 }
 
-inline double planar_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb)
+// Vectors per thread of the planar kernel when it takes several at once.
+inline int planar_vb(int storage, int nvec)
 {
-    const double sites = (double)nblk * g.Vs;
-    const double site = nvec == 2 ? 0.06 : nvec == 3 ? 0.108 : 0.132;
-    const double l2 = sites * (3.0 * wb + 2.0 * vby * nvec) < 60e6 ? 0.7 : 1.0;  // stays in L2
-    return sites * site * l2 * (wb == 48 ? 1.15 : 1.0) * (vby == 16 ? 0.9 : 1.0) * 1e-3 + 2.5;
+    const int cap = storage == P_F64 ? 4 : 8;
+    int vb = 2;
+    while (vb < cap && vb < nvec) vb *= 2;
+    return vb;
+}
+
+// All vectors in one launch of the planar kernel, two or four a thread: reads W once, has no rows
+// to keep whole, but pays for unused lanes of its four vectors.  For two to four vectors; not for
+// the 8-real W, whose reconstruction rounds differently there.
+inline double planar_estimate(const SubGeom &g, int nblk, int nvec, int vby, int wb, int num_sms)
+{
+    static const double per_warp[SF_N][2] = {{.254, .523}, {.317, .585}, {0, 0}, {.298, .468}, {.273, .473}, {.246, .456}};
+    if (wb == 32 || nvec < 2 || nvec > 4) return 1e300;
+    const double warps = (double)(((int64_t)nblk * g.Vs + 31) / 32);
+    const double a = per_warp[step_fmt(vby, wb)][nvec > 2] * warps / num_sms, b = 1.6 * nvec;
+    return 2.5 + 1.07 * std::pow(std::pow(a, 1.46) + std::pow(b, 1.46), 1 / 1.46);
+}
+
+// What the fit of col_estimate leaves out when kernels are compared, from the same 1600 problems
+// (spread 15 %): tiles of one or two warps and 16-bit records take longer, W f32-8 less.
+inline double col_bias(const ColPlan &p, int vby, int wb)
+{
+    return (p.threads <= 32 ? 1.34 : p.threads <= 64 ? 1.12 : 1.0) * (vby == 16 ? 1.075 : 1.0) * (wb == 32 ? 0.9 : 1.0);
 }
 
 // The best tile shapes by that estimate, best first (at most `most`).  nvg divides
@@ -219,6 +312,58 @@ inline int col_plans(const SubGeom &g, int nblk, int nvec, int vby, int wb, int 
     return n;
 }
 
+// tile[] of the tune entry for a shape: 9 selects the column kernel.
+inline void col_tile_of(const ColPlan &p, int tile[3])
+{
+    tile[0] = p.nvg;
+    tile[1] = 9;
+    tile[2] = p.ny | p.nseg << 8 | p.units << 16;
+}
+
+// The kernel of a call without a tune entry: the cheapest by these estimates.  The plain kernel gets
+// 5 % of credit, it was the only one before the others came in: chosen by earlier estimates,
+// which knew neither it nor rows off 16 bytes, 266 of the 1600 problems ran more than 10 % slower
+// than with it (up to 2.0 times), now 10 (up to 1.3); the mean over all is 1.32 times its rate, 1.26
+// before.
+enum StepKind { STEP_IL, STEP_ROW, STEP_COL, STEP_PLANAR };
+
+struct StepPlan {
+    int kind, vb;  // vb 0: the kernel's own rule
+    int tile[3];
+    ColPlan col;
+};
+
+// n of the call's nvec vectors are packed at a time; exact: no padded groups; planar: the planar kernel
+// is possible.
+inline StepPlan plan_step(const SubGeom &g, int nblk, int nvec, int n, int vby, int wb, int num_sms, bool exact, bool planar)
+{
+    StepPlan s{};
+    const int n2 = (n + 1) & ~1;
+    double best = 0.95 * il_estimate(g, nblk, n2, vby, wb, num_sms);
+    s.kind = STEP_IL;
+    const double row = row_estimate(g, nblk, n2, vby, wb, num_sms);
+    if (row < best) {
+        best = row;
+        s.kind = STEP_ROW;
+    }
+    const double pl = planar ? planar_estimate(g, nblk, nvec, vby, wb, num_sms) : 1e300;
+    if (pl < best) {
+        best = pl;
+        s.kind = STEP_PLANAR;
+    }
+    double us = 0;
+    if (col_plans(g, nblk, exact ? n2 : n, vby, wb, num_sms, &s.col, &us, 1, exact) > 0 &&
+        us * col_bias(s.col, vby, wb) < best)
+        s.kind = STEP_COL;
+    if (s.kind == STEP_ROW) s.vb = row_tile(g, nblk, n, vby, s.tile);
+    if (s.kind == STEP_PLANAR) s.tile[1] = 10;
+    if (s.kind == STEP_COL) {
+        s.vb = 2;
+        col_tile_of(s.col, s.tile);
+    }
+    return s;
+}
+
 // Whether buffers of have[k] bytes can grow to need[k] under an HBM cap (0: none) with `used` bytes
 // in use, the old ones counted.  Known before a buffer is given up: a call that tried the padded
 // groups of the column kernel and failed freed, allocated and cleared its buffers each time.
@@ -229,44 +374,10 @@ inline bool workspace_fits(uint64_t used, uint64_t cap, int n, const uint64_t *h
     return cap == 0 || used <= cap;
 }
 
-// tile[] of the tune entry for a shape: 9 selects the column kernel.
-inline void col_tile_of(const ColPlan &p, int tile[3])
-{
-    tile[0] = p.nvg;
-    tile[1] = 9;
-    tile[2] = p.ny | p.nseg << 8 | p.units << 16;
-}
-
 // The shape of such an entry.  False: no fit.
 inline bool col_of_tile(const SubGeom &g, int nblk, int nvec, int vby, int wb, const int tile[3], ColPlan &out)
 {
     return col_shape(g, nblk, nvec, vby, wb, tile[0], tile[2] & 255, std::max(1, (tile[2] >> 8) & 255), tile[2] >> 16, out);
-}
-
-// Row kernel parameters without a tune entry: tile[], returns the vectors per thread.
-// More than 24 vectors go through CTAs of 24 where that divides them (72 vectors at
-// 48^3 x 24: 2.41 ms against 2.64 with 36 a CTA); rows are asked into L2 ahead (tile[2])
-// where a step's data do not stay there (64^3 x 24, 24 vectors: 1.61 against 1.64 ms;
-// 16^3 x 32, 2 vectors: 21 against 19 us).  Four vectors per thread where the rows then still
-// fill a warp (32^3 x 64 / 48^3 x 32, 3 vectors: 16 / 24 threads, 180 / 224 us with four and
-// 142 / 290 with two); 16-bit records want twice the threads (12 vectors, 48 threads: 434
-// against 369 us; 24 vectors, 144 threads: 1203 against 1507).
-inline int row_tile(const SubGeom &g, int nblk, int nvec, int vby, int tile[3])
-{
-    const int n = (nvec + 1) & ~1;
-    tile[0] = n > 24 && n % 24 == 0 ? 24 : 0;
-    tile[1] = 6;
-    tile[2] = (double)nblk * g.Vs * (216.0 + 2.0 * vby * n) > 120e6 ? -1 : 0;
-    return n % 4 == 0 && n / 4 * g.hx >= (vby == 16 ? 64 : 20) ? 4 : 2;
-}
-
-// Vectors per thread of the planar kernel when it takes several at once.
-inline int planar_vb(int storage, int nvec)
-{
-    const int cap = storage == P_F64 ? 4 : 8;
-    int vb = 2;
-    while (vb < cap && vb < nvec) vb *= 2;
-    return vb;
 }
 
 // Share of the lanes of a warp at work in the FP64 multi-RHS kernel (nvec threads per site, a

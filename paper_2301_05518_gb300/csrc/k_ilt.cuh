@@ -43,23 +43,13 @@
 // more (bounded) for its own copies in flight and returns without writing.
 #pragma once
 
+#include "col_plan.h"
 #include "launch.cuh"
 #include "tls_dev.cuh"
 #include "tls_internal.h"
 #include "tma.cuh"
 
 namespace tls {
-
-// Shared-memory bytes of the k_step_ilt CTA: the mbarrier (128 bytes) and the five W rows.
-inline int ilt_smem(int hx, int wb) { return 128 + 5 * hx * wb; }
-
-// Whether the TMA staging applies: every plane segment of a W row starts and
-// ends on a 16-byte boundary (the remainder plane has 4 or 8 bytes per site).
-inline bool ilt_ok(int wfmt, const SubGeom &g)
-{
-    const int rem = wfmt_bytes(wfmt) % 16;
-    return rem == 0 || (g.hx * rem) % 16 == 0;
-}
 
 // Issues the bulk copies of the five W rows of row (blk, zq, yq) into the
 // sets at ws (one elected thread); completion lands on bar.
@@ -657,17 +647,6 @@ __global__ void __launch_bounds__(MAXT, MINB) k_step_ilt(const char *__restrict_
     if (st.any) st.compute(ws, g.hx, k, t, T, alphaf);
 }
 
-// Vectors per CTA: tile[0] if it is a multiple of VB dividing nvec, else the
-// largest such count with (count / VB) * hx <= 256 threads.  0: no fit.
-inline int ilt_group(int nvec, int vb, int hx, int want)
-{
-    auto fits = [&](int n) { return n >= vb && n % vb == 0 && nvec % n == 0 && (n / vb) * hx <= 256; };
-    if (want > 0 && fits(want)) return want;
-    for (int n = nvec; n >= vb; n -= vb)
-        if (fits(n)) return n;
-    return 0;
-}
-
 // tile[1] = 6: registers capped for 3 CTAs of 256 threads per SM; 7: the next
 // hop's records prefetched, registers for 3 CTAs of 192 threads (2 of 256
 // when the row needs more threads); 8: the row's own records staged with the
@@ -678,14 +657,14 @@ template <int VP, int WF, int VB> cudaError_t ilt_launch(const StepArgs &a)
     if constexpr (VP == P_F64 || (VB > 4 && !(VP == P_F32 && VB == 8))) {
         return cudaErrorNotSupported;
     } else {
-        if (!a.err || !a.alphaf || !ilt_ok(WF, a.g)) return cudaErrorNotSupported;
-        const int nvg = ilt_group(a.nvec, VB, a.g.hx, a.tile[0]);
+        if (!a.err || !a.alphaf || !row_tma(a.g.hx, wfmt_bytes(WF))) return cudaErrorNotSupported;
+        const int nvg = row_group(a.nvec, VB, a.g.hx, a.tile[0]);
         if (nvg == 0) return cudaErrorNotSupported;
         dim3 block(nvg / VB, a.g.hx);
         dim3 grid(a.nvec / nvg, a.g.hy, (unsigned)a.g.hz * a.nblk);
         if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-        const int smem = ilt_smem(a.g.hx, wfmt_bytes(WF));
-        if (smem > (48 << 10)) return cudaErrorNotSupported;
+        const int smem = row_smem(a.g.hx, wfmt_bytes(WF));
+        if (smem > kRowMaxSmem) return cudaErrorNotSupported;
         const bool act = a.active != nullptr;
         const int threads = block.x * block.y;
         // L2 prefetch distance in planes: tile[2] > 0 as given, 0 none, < 0

@@ -1042,17 +1042,6 @@ template <int VP, int WF, int VB> int persist_occ(int threads)
     return n;
 }
 
-// Sites per CTA for the interleaved kernels: nvec * spb <= threads, with a
-// whole number of warps when possible.
-inline int il_spb(int nvec, int threads)
-{
-    if (threads <= 0) threads = 256;
-    int spb = std::max(1, threads / nvec);
-    for (int s = spb; s >= 1; --s)
-        if ((s * nvec) % 32 == 0) return s;
-    return spb;
-}
-
 // ONLYX: only the packed FP32 pair kernel is instantiated (eight vectors per thread).
 template <int VP, int WF, int VB, bool ONLYX = false> cudaError_t step_il_launch(const StepArgs &a)
 {

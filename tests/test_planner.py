@@ -41,6 +41,12 @@ double estimate(const int *h, int nblk, int nvec, int vby, int wb, const int *ti
     ColPlan p;
     return col_of_tile(geom(h), nblk, nvec, vby, wb, tile, p) ? col_estimate(p, geom(h), nblk, vby, wb, 152, 1e300) : 1e300;
 }
+int planned(const int *h, int nblk, int nvec, int vby, int wb, int exact, int planar, int *tile)
+{
+    const StepPlan s = plan_step(geom(h), nblk, nvec, nvec, vby, wb, 152, exact, planar);
+    for (int k = 0; k < 3; ++k) tile[k] = s.tile[k];
+    return s.kind;
+}
 void split(int T, int Lx, int nrow, int *o)
 {
     const PairSplit p = pair_split(T, Lx, nrow);
@@ -153,3 +159,42 @@ def test_search_finds_the_best_shapes(plan, h, nblk, nvec, vby, wb):
     for k in range(n):
         t = tuple(tiles[3 * k:3 * k + 3])
         assert t in every and plan.estimate(ints(*h), nblk, nvec, vby, wb, ints(*t)) == times[k]
+
+
+IL, ROW, COL, PLANAR = range(4)
+
+
+# measured us per step (interleaved / row or its stand-in / column / planar), a GB300: kernels within 10 % of the best
+@pytest.mark.parametrize("h,nblk,nvec,vby,wb,good", [
+    ((22, 22, 22), 8, 26, 24, 48, {IL, COL}),      # 51 / 103 / 48: the row kernel is left one pair a CTA
+    ((13, 2, 21), 336, 46, 24, 32, {IL}),          # 293 / 567 / 508
+    ((17, 17, 17), 8, 4, 24, 72, {IL, COL}),       # 8.2 / 14.5 / 8.7 / 11.1: rows off 16 bytes
+    ((13, 13, 13), 264, 53, 16, 24, {IL}),         # 609 / 732 / 791
+    ((29, 29, 29), 40, 6, 16, 24, {IL}),           # 119 / 181 / 154 / 255
+    ((24, 24, 24), 512, 24, 24, 72, {COL}),        # 3980 / 1950 / 1800
+    ((32, 32, 32), 128, 24, 24, 48, {ROW, COL}),   # 2126 / 1188 / 1232
+    ((16, 16, 16), 256, 24, 24, 32, {ROW}),        # 573 / 450
+    ((8, 8, 8), 8, 6, 16, 36, {ROW}),              # 6.1 / 2.8 / 10.4
+    ((14, 14, 14), 40, 2, 24, 72, {ROW, PLANAR}),  # 12.7 / 9.5 / 16.0 / 8.1
+])
+def test_planned_kernel_is_a_good_one(plan, h, nblk, nvec, vby, wb, good):
+    assert plan.planned(ints(*h), nblk, nvec, vby, wb, 0, 1, ints(0, 0, 0)) in good
+
+
+@pytest.mark.parametrize("vby,wb", [(24, 72), (24, 48), (24, 32), (16, 72), (16, 48), (16, 36), (16, 24)])
+def test_plan_is_launchable(plan, vby, wb):
+    """Over sizes and counts: a planned column shape fits as it is written down, padded groups only where
+    they are allowed, the planar kernel only where it is possible."""
+    for h in ((1, 1, 1), (1, 300, 2), (3, 7, 5), (17, 4, 9), (24, 24, 24), (150, 3, 2)):
+        for nblk in (1, 8, 200):
+            for nvec in (1, 2, 3, 5, 24, 31, 96, 256):
+                for exact in (0, 1):
+                    t = ints(0, 0, 0)
+                    kind = plan.planned(ints(*h), nblk, nvec, vby, wb, exact, 0, t)
+                    assert kind in (IL, ROW, COL)
+                    if kind == COL:
+                        o = ints(*[0] * 7)
+                        assert t[1] == 9 and plan.entry_shape(ints(*h), nblk, nvec, vby, wb, t, o) == 1
+                        assert not exact or ((nvec + 1) & ~1) % t[0] == 0
+                    else:
+                        assert t[1] == (6 if kind == ROW else 0)
