@@ -697,6 +697,16 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
     const size_t io_elem = io_prec == TLS_F64 ? 8 : 4;
     const size_t io_slice_bytes = (size_t)Vslice * 6 * io_elem;
 
+    // Host vectors go through slice groups of about kGroupBytes in up to three rotating staging
+    // slots, so that copies in and out overlap the smearing of other groups.
+    const bool staged = !vecs_on_device;
+    int tg = nsl;  // slices of a group
+    if (staged && nsl >= 2) {
+        const size_t total = io_slice_bytes * nsl * nvec;
+        const int64_t want = std::max<int64_t>(4, (int64_t)((total + kGroupBytes - 1) / kGroupBytes));
+        tg = (int)((nsl + std::min<int64_t>(nsl, want) - 1) / std::min<int64_t>(nsl, want));
+    }
+
     // Kernel choice: explicit kernel, or the autotune table, or the planner.
     int kern = kernel;
     int vb = 0;
@@ -708,9 +718,12 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         auto it = ctx->tune.find(key);
         const bool have = it != ctx->tune.end();
         if (kern == TLS_KERNEL_AUTO) {
-            kern = have ? it->second.kernel
-                   : nvec == 1 || (storage == TLS_F64 && op == 0 && il_f64_lanes(nvec, g.hx) < 0.97) ? TLS_KERNEL_SINGLE
-                                                                                                    : TLS_KERNEL_MRHS;
+            const int nb = tg * bps;
+            kern = have         ? it->second.kernel
+                   : nvec == 1 || (storage == TLS_F64 && op == 0 && f64_single_estimate(g, nb, nvec, ctx->num_sms) <
+                                                                        f64_il_estimate(g, nb, nvec, ctx->num_sms))
+                       ? TLS_KERNEL_SINGLE
+                       : TLS_KERNEL_MRHS;
         }
         if (have && it->second.kernel == kern) {
             vb = it->second.vb;
@@ -741,22 +754,10 @@ tls_status smear_impl(tls_ctx *ctx, tls_gauge_id id, void *vecs, int io_prec, in
         col = col_of_tile(g, nblk, col_n, VBY, wfmt_bytes(fmt), tile, cp);
         planned = !col;
     }
-    // Host vectors go through slice groups of about kGroupBytes in up to three
-    // rotating staging slots, so that copies in and out overlap the smearing
-    // of other groups.  The persistent kernel takes all slices in one group.
-    const bool staged = !vecs_on_device;
-    int tg = nsl, ngroup = 1, nslot = 1;
-    size_t slot_bytes = 0;
-    if (staged) {
-        const size_t total = io_slice_bytes * nsl * nvec;
-        if (kern != TLS_KERNEL_PERSISTENT && nsl >= 2) {
-            const int64_t want = std::max<int64_t>(4, (int64_t)((total + kGroupBytes - 1) / kGroupBytes));
-            tg = (int)((nsl + std::min<int64_t>(nsl, want) - 1) / std::min<int64_t>(nsl, want));
-            ngroup = (nsl + tg - 1) / tg;
-        }
-        nslot = std::min(ngroup, 3);
-        slot_bytes = (io_slice_bytes * tg * nvec + 255) / 256 * 256;
-    }
+    // The persistent kernel takes all slices in one group.
+    if (kern == TLS_KERNEL_PERSISTENT) tg = nsl;
+    const int ngroup = (nsl + tg - 1) / tg, nslot = std::min(ngroup, 3);
+    const size_t slot_bytes = (io_slice_bytes * tg * nvec + 255) / 256 * 256;
     auto plan = [&](bool exact) {  // for the slices of one launch
         const StepPlan p = plan_step(g, tg * bps, nvec, col_n, VBY, wfmt_bytes(fmt), ctx->num_sms, exact, op == 0);
         col = p.kind == STEP_COL;

@@ -380,23 +380,36 @@ inline bool col_of_tile(const SubGeom &g, int nblk, int nvec, int vby, int wb, c
     return col_shape(g, nblk, nvec, vby, wb, tile[0], tile[2] & 255, std::max(1, (tile[2] >> 8) & 255), tile[2] >> 16, out);
 }
 
-// Share of the lanes of a warp at work in the FP64 multi-RHS kernel (nvec threads per site, a
-// strip of one row per CTA of at most 256 threads).  The FP64 pipe bounds it, so idle lanes cost
-// their share, and one vector per launch, which has none, reads W more often for nothing lost
-// (32^3 x 16, 3 vectors: 48 of 64 lanes, 779 us per step against 597; 4 vectors: 779 against 796).
-inline double il_f64_lanes(int nvec, int hx)
+// FP64 steps.  The FP64 pipe of an SM takes 1.82 us for the step of a warp (32 sites and vectors),
+// so what counts is the warps on the busiest SM, beside what a launch costs; fitted to 110 measured
+// problems (one slice of 8^3 to 48^3, 8^3 x 8 to 32^3 x 16, odd rows, 2 to 30 vectors), within 10 %.
+// One launch per vector and step: small lattices run three threads a site in CTAs of one warp.
+inline double f64_single_estimate(const SubGeom &g, int nblk, int nvec, int num_sms)
 {
-    const int n = nvec < 256 ? nvec : 256;
-    int spb = std::max(1, 256 / n);
-    for (int s = spb; s >= 1; --s)
-        if ((s * n) % 32 == 0) {
-            spb = s;
-            break;
-        }
-    spb = std::min(spb, hx);
-    const int strips = (hx + spb - 1) / spb;  // the last one may be short, its CTA is not
-    const double threads = (double)strips * ((spb * n + 31) / 32 * 32);
-    return (double)hx * n / threads;
+    const int64_t sites = (int64_t)nblk * g.Vs;
+    auto per_sm = [&](int64_t n) { return (double)((n + num_sms - 1) / num_sms); };
+    const int64_t rows = (sites + 31) / 32 * 3;
+    const double one = sites > (int64_t)4 * 32 * num_sms ? 3 + 1.82 * 4 * per_sm((sites + 127) / 128)
+                       : rows <= 2 * num_sms             ? 4.2
+                                                         : std::max(9.3, 3 + 0.62 * per_sm(rows));
+    return nvec * one;
+}
+
+// All vectors in one launch (k_step_il, one vector a thread): strips of a row, whose last one may be
+// short.  Idle lanes cost their share (32^3 x 16, 3 vectors: 48 of 64 lanes, 778 us against 598
+// one by one), launches theirs (8^3, one slice, 12 vectors: 12.6 us against 47.7).
+inline double f64_il_estimate(const SubGeom &g, int nblk, int nvec, int num_sms)
+{
+    double us = 0;
+    for (int v = 0; v < nvec; v += 256) {
+        const int n = std::min(nvec - v, 256), spb = std::min(il_spb(n, 256), g.hx);
+        const int full = g.hx / spb, rest = g.hx - full * spb;
+        const double warps = (double)full * ((spb * n + 31) / 32) + (rest * n + 31) / 32;  // of a row
+        const int strips = full + (rest > 0);
+        const int64_t ctas = (int64_t)strips * g.hy * g.hz * nblk;
+        us += std::max(12.4, 4 + 1.82 * ((ctas + num_sms - 1) / num_sms) * warps / strips);
+    }
+    return us;
 }
 
 }  // namespace tls

@@ -47,6 +47,10 @@ int planned(const int *h, int nblk, int nvec, int vby, int wb, int exact, int pl
     for (int k = 0; k < 3; ++k) tile[k] = s.tile[k];
     return s.kind;
 }
+double f64_us(const int *h, int nblk, int nvec, int single)
+{
+    return single ? f64_single_estimate(geom(h), nblk, nvec, 152) : f64_il_estimate(geom(h), nblk, nvec, 152);
+}
 void split(int T, int Lx, int nrow, int *o)
 {
     const PairSplit p = pair_split(T, Lx, nrow);
@@ -69,7 +73,7 @@ def plan(tmp_path_factory):
     subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I" + CSRC, "-o", str(d / "plan.so"),
                            str(d / "glue.cpp")])
     lib = ctypes.CDLL(str(d / "plan.so"))
-    lib.estimate.restype = ctypes.c_double
+    lib.estimate.restype = lib.f64_us.restype = ctypes.c_double
     return lib
 
 
@@ -198,3 +202,28 @@ def test_plan_is_launchable(plan, vby, wb):
                         assert not exact or ((nvec + 1) & ~1) % t[0] == 0
                     else:
                         assert t[1] == (6 if kind == ROW else 0)
+
+
+# half extents, blocks, then vectors and measured us per step: one launch per vector / one for all
+F64 = [
+    ((4, 4, 4), 8, [(2, 7.9, 12.4), (3, 12.1, 12.5), (6, 23.9, 12.4), (12, 47.7, 12.6), (24, 95.5, 12.6), (30, 119.5, 12.5)]),
+    ((6, 6, 6), 8, [(2, 8.0, 12.4), (3, 12.3, 12.5), (6, 24.6, 12.5), (12, 52.0, 14.5), (24, 107.8, 22.8), (30, 140.7, 25.0)]),
+    ((8, 8, 8), 8, [(2, 17.3, 12.6), (3, 27.2, 12.3), (6, 55.4, 18.6), (12, 110.9, 24.8), (24, 221.3, 47.4), (30, 276.2, 61.8)]),
+    ((12, 12, 12), 8, [(2, 19.1, 18.8), (3, 28.8, 33.1), (6, 57.5, 47.4), (12, 114.6, 76.2), (24, 228.9, 140.5), (30, 286.1, 176.7)]),
+    ((16, 16, 16), 128, [(2, 399.2, 392.3), (3, 598.4, 778.1), (6, 1195.4, 1164.5), (12, 2391.1, 2322.2), (24, 4780.5, 4636.6), (30, 5977.0, 6177.9)]),
+    ((4, 4, 4), 64, [(2, 17.1, 16.4), (3, 26.9, 16.4), (6, 55.2, 16.4), (12, 110.6, 30.8), (24, 220.3, 43.2), (30, 275.6, 53.6)]),
+    ((24, 24, 24), 8, [(2, 94.6, 119.6), (3, 141.9, 176.7), (6, 283.1, 283.2), (12, 566.2, 505.9), (24, 1131.5, 983.1), (30, 1414.1, 1308.6)]),
+    ((8, 8, 8), 64, [(2, 37.4, 53.6), (3, 55.8, 53.7), (6, 111.2, 104.7), (12, 221.6, 154.1), (24, 442.7, 295.3), (30, 553.1, 391.9)]),
+    ((3, 5, 7), 32, [(2, 15.0, 18.7), (3, 26.0, 18.9), (6, 56.5, 18.7), (12, 113.6, 33.1), (24, 227.0, 47.5), (30, 282.9, 47.6)]),
+    ((6, 6, 6), 192, [(2, 50.9, 90.6), (3, 76.7, 90.7), (6, 154.1, 168.8), (12, 306.7, 252.6), (24, 613.7, 417.7), (30, 766.4, 498.2)]),
+]
+
+
+@pytest.mark.parametrize("h,nblk,times", F64)
+def test_f64_choice(plan, h, nblk, times):
+    """One FP64 vector per launch or all in one: the choice is within 10 % of the better one (a launch's
+    time: within 5 us)."""
+    for nvec, single, together in times:
+        a, b = plan.f64_us(ints(*h), nblk, nvec, 1), plan.f64_us(ints(*h), nblk, nvec, 0)
+        chosen = single if a < b else together
+        assert chosen <= max(1.1 * min(single, together), min(single, together) + 5), (nvec, a, b, single, together)
