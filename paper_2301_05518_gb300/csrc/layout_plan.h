@@ -30,6 +30,16 @@ inline PairSplit pair_split(int T, int Lx, int nrow)
     return p;
 }
 
+// Rows of a CTA that takes short rows of links together (an even number), 0: a row by itself, the
+// better form from eight sites up (load and release, us, by itself / together: 2 x 96 x 96 x 96 1676 /
+// 998, 4 x 64 x 64 x 64 709 / 576, 6 x 64 x 64 x 48 763 / 699, 8 x 32 x 32 x 32 262 / 266, 16 x 48 x 48 x
+// 32 661 / 697) and where few CTAs are left (2 x 8 x 8 x 8 26.6 / 30.5).
+inline int ingest_rows(int Lx, int sites, int64_t nrow)
+{
+    const int rows = sites / Lx & ~1;
+    return Lx <= 6 && nrow >= (int64_t)304 * rows ? rows : 0;
+}
+
 // Strided subsets of a part of a slice's norm, `split` or one: by the slice alone, since it sets the
 // order of the additions.  From 28^3 sites on a thread of `split` CTAs has eight reals or more.
 inline int norm_subsets(int64_t slice_sites, int split) { return slice_sites * 6 >= 131072 ? split : 1; }

@@ -51,6 +51,7 @@ double f64_us(const int *h, int nblk, int nvec, int single)
 {
     return single ? f64_single_estimate(geom(h), nblk, nvec, 152) : f64_il_estimate(geom(h), nblk, nvec, 152);
 }
+int link_rows(int Lx, long long nrow) { return ingest_rows(Lx, 64, nrow); }
 void split(int T, int Lx, int nrow, int *o)
 {
     const PairSplit p = pair_split(T, Lx, nrow);
@@ -227,3 +228,9 @@ def test_f64_choice(plan, h, nblk, times):
         a, b = plan.f64_us(ints(*h), nblk, nvec, 1), plan.f64_us(ints(*h), nblk, nvec, 0)
         chosen = single if a < b else together
         assert chosen <= max(1.1 * min(single, together), min(single, together) + 5), (nvec, a, b, single, together)
+
+
+@pytest.mark.parametrize("Lx,nrow,want", [(2, 110592, 32), (4, 55296, 16), (6, 100000, 10), (8, 100000, 0), (48, 100000, 0),
+                                          (2, 512, 0), (2, 304 * 32, 32), (2, 304 * 32 - 2, 0)])
+def test_short_rows_of_links_share_a_cta(plan, Lx, nrow, want):
+    assert plan.link_rows(Lx, ctypes.c_longlong(nrow)) == want
