@@ -320,9 +320,9 @@ inline void col_tile_of(const ColPlan &p, int tile[3])
     tile[2] = p.ny | p.nseg << 8 | p.units << 16;
 }
 
-// The kernel of a call without a tune entry: the cheapest by these estimates.  The plain kernel gets
-// 5 % of credit, it was the only one before the others came in: chosen by earlier estimates,
-// which knew neither it nor rows off 16 bytes, 266 of the 1600 problems ran more than 10 % slower
+// The kernel of a call without a tune entry: the cheapest by these estimates.  In short steps, where
+// they are least sure, the plain kernel gets 5 % of credit: it was the only one before the others
+// came in.  Chosen by earlier estimates, which knew neither it nor rows off 16 bytes, 266 of the 1600 problems ran more than 10 % slower
 // than with it (up to 2.0 times), now 10 (up to 1.3); the mean over all is 1.32 times its rate, 1.26
 // before.
 enum StepKind { STEP_IL, STEP_ROW, STEP_COL, STEP_PLANAR };
@@ -339,7 +339,8 @@ inline StepPlan plan_step(const SubGeom &g, int nblk, int nvec, int n, int vby, 
 {
     StepPlan s{};
     const int n2 = (n + 1) & ~1;
-    double best = 0.95 * il_estimate(g, nblk, n2, vby, wb, num_sms);
+    double best = il_estimate(g, nblk, n2, vby, wb, num_sms);
+    if (best < 40) best *= 0.95;
     s.kind = STEP_IL;
     const double row = row_estimate(g, nblk, n2, vby, wb, num_sms);
     if (row < best) {
