@@ -23,11 +23,10 @@ struct Cand {
 
 std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, int num_sms, bool exact)
 {
-    // The kernels that won at some measured shape.  Measured and dropped (they
-    // never won at any benchmarked shape): the register-capped and W-staged
-    // interleaved variants, explicit strip lengths, eight vectors per thread, the
-    // row kernel with the next hop's records requested early, the TMA row kernel, the z-marching kernel and both
-    // persistent forms (tls_smear still runs any of them when asked for).
+    // The kernels that won at some measured shape.  Measured and dropped (they never won at
+    // any benchmarked shape): the register-capped and W-staged interleaved variants, explicit strip
+    // lengths, the TMA row kernel, the z-marching kernel and both persistent forms (tls_smear
+    // still runs any of them when asked for).
     std::vector<Cand> c;
     if (nvec <= 4) {
         c.push_back({TLS_KERNEL_SINGLE, 1, 128, {0, 0, 0}});
@@ -40,9 +39,13 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
         // under an HBM cap only groups without padding, as the planner does
         const int n = col_plans(gg.g, nsl * 8, exact ? (G + 1) & ~1 : G, vfmt_bytes(storage), wfmt_bytes(gg.wfmt), num_sms,
                                 best, us, 3, exact);
+        const int vby = vfmt_bytes(storage), wb = wfmt_bytes(gg.wfmt), G2 = (G + 1) & ~1;
+        const double row = row_estimate(gg.g, nsl * 8, G2, vby, wb, num_sms);
         if (nvec >= 2 && nvec <= 4 && gg.wfmt != W_F32_8)  // planar vectors in one launch
             c.push_back({TLS_KERNEL_MRHS, planar_vb(storage, nvec), 128, {0, 10, 0}});
+        c.push_back({TLS_KERNEL_MRHS, default_il_vb(storage, G2), 256, {0, 0, 0}});  // no staging: any row
         for (int k = 0; k < n; ++k) {
+            if (us[k] * col_bias(best[k], vby, wb) > 1.3 * row) continue;  // out of reach of the estimate's error
             Cand cd{TLS_KERNEL_MRHS, 2, 0, {0, 0, 0}};
             col_tile_of(best[k], cd.tile);
             c.push_back(cd);
@@ -60,6 +63,10 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
         // whole rows with the W rows staged by TMA: all vectors or half of them per CTA
         c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 6, 0}});
         c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 6, -1}});  // rows ahead requested into L2
+        // the next hop's records requested early: wins with W f32-12 and f32-8 and on small slices (48^3 x
+        // 64, 24 vectors, f32-12: 2060 us against 2072 with the column kernel; 32^3 x 32, 16 vectors:
+        // 193 against 201)
+        c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 7, 0}});
         if (vb % 2 == 0) c.push_back({TLS_KERNEL_MRHS, vb, 0, {0, 8, 0}});  // the row's records staged too
         // fewer vectors per CTA: smaller CTAs, W staged once per group (each
         // distinct count once)
@@ -72,6 +79,11 @@ std::vector<Cand> candidates(int nvec, int storage, const Gauge &gg, int nsl, in
         }
         // packed FP32 pairs with the W broadcasts staged by the threads (any row length)
         c.push_back({TLS_KERNEL_MRHS, vb, 128, {0, 2, 0}});
+    }
+    if (storage == TLS_F32 && G2 % 8 == 0 && gg.wfmt != W_F32_18) {  // eight vectors share W's reconstruction
+        c.push_back({TLS_KERNEL_MRHS, 8, 0, {0, 6, 0}});
+        c.push_back({TLS_KERNEL_MRHS, 8, 0, {0, 7, 0}});
+        c.push_back({TLS_KERNEL_MRHS, 8, 0, {0, 7, -1}});
     }
     return c;
 }
