@@ -294,8 +294,9 @@ typedef struct {
                             /* take tile[1] = 2); 9 marches tiles of rows      */
                             /* along z (FP32 and 16-bit storage): tile[0] =    */
                             /* vectors per group (even), tile[2] = rows per    */
-                            /* tile | z segments << 8 | ring units << 16 (a    */
-                            /* shape that does not fit goes to the planner);   */
+                            /* tile | z segments << 8 | ring units << 16 (0 or */
+                            /* from 3 up; a shape that does not fit goes to    */
+                            /* the planner);                                   */
                             /* 10 keeps planar vectors, up to 8 in one launch; */
                             /* tile[2] (tile[1] = 6..8): each CTA requests     */
                             /* into L2 the W rows and records of the row       */
